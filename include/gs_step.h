@@ -105,14 +105,17 @@ typedef struct {
                                  (Gaussian, pixel block) pairs summing them
                                  (the paper's second implementation) */
     int32_t threads_per_tile; /* threads of a raster_bwd thread block
-                                 (bwd_impl 0): 0 or tile_w x tile_h = one per
-                                 pixel; half or (16-wide tiles) a quarter of
-                                 that = 2 or 4 pixels per thread, each warp
-                                 covering 8 x 8 or 8 x 16 pixels (Sec. 4.2: the
-                                 scheduler's threads per tile).  Pixels per
-                                 thread other than 1 need bwd_impl 0.  The
-                                 raster forward always runs one thread per
-                                 pixel. */
+                                 (bwd_impl 0): 0 or tile_w x tile_h = the sums
+                                 of one pixel per thread; half or (16-wide
+                                 tiles) a quarter of that = 2 or 4 pixels per
+                                 thread, each warp covering 8 x 8 or 8 x 16
+                                 pixels (Sec. 4.2: the scheduler's threads per
+                                 tile).  Pixels per thread other than 1 need
+                                 bwd_impl 0.  It selects how the gradient sums
+                                 are formed; the library maps one pixel per
+                                 thread (and two, with BF16 moments) to lane
+                                 groups over 8 x 4 pixel blocks.  The raster
+                                 forward does not depend on it. */
 } gs_tuning;
 
 typedef struct {

@@ -17,19 +17,25 @@
 namespace gs {
 
 // ---- packed FP32 pairs: each half is one correctly rounded operation, the
-// same bits as the scalar form, at half the issue slots
+// same bits as the scalar form, at half the issue slots.  Written with the
+// explicit rounding, which keeps a product and a sum from being fused.
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+
+#define GS_PACKED2(name, op)                                                                                   \
+    __device__ __forceinline__ float2 name(float2 a, float2 b)                                                 \
+    {                                                                                                          \
+        unsigned long long d;                                                                                  \
+        asm(op ".rn.f32x2 %0, %1, %2;"                                                                         \
+            : "=l"(d)                                                                                          \
+            : "l"(*reinterpret_cast<unsigned long long*>(&a)), "l"(*reinterpret_cast<unsigned long long*>(&b))); \
+        return *reinterpret_cast<float2*>(&d);                                                                 \
+    }
+GS_PACKED2(mul2, "mul")
+GS_PACKED2(add2, "add")
+GS_PACKED2(sub2, "sub")
+#undef GS_PACKED2
+
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b)
-{
-    unsigned long long d;
-    asm("sub.rn.f32x2 %0, %1, %2;"
-        : "=l"(d)
-        : "l"(*reinterpret_cast<unsigned long long*>(&a)), "l"(*reinterpret_cast<unsigned long long*>(&b)));
-    return *reinterpret_cast<float2*>(&d);
-}
 
 // ---- geometry of the blocks of a TW x TH tile
 template <int TW, int TH>
@@ -50,10 +56,10 @@ struct TileBlocks {
     }
 };
 
-// Conservative mask of the tile's 4x4 blocks that an entry can contribute
-// to; warp w's four blocks are the bits 4w .. 4w + 3 (lane group g = bit
-// 4w + g).  (x, y): the mean relative to the centre of the tile's first
-// pixel.  A pair needs d^2 <= r^2 = min(9, 2 ln(255 o)); for each row of blocks
+// Conservative mask of the tile's BW x 4 blocks (BW = 4 or 8) that an entry can
+// contribute to; warp w's four blocks are the bits 4w .. 4w + 3 (lane group
+// g = bit 4w + g): 4x4 blocks in quads of 8x8 pixels, 8x4 blocks row by row.
+// (x, y): the mean relative to the centre of the tile's first pixel.  A pair needs d^2 <= r^2 = min(9, 2 ln(255 o)); for each row of blocks
 // the ellipse's extreme x over the row's band gives the first and last block:
 // with h(dy) = sqrt(r^2/a - det dy^2 / a^2) the ellipse spans
 // x - (b/a) dy -/+ h(dy), extreme at dy = -/+ ys (the offset of the leftmost /
@@ -64,11 +70,11 @@ struct TileBlocks {
 // kappa = a c / det, which bounds the rounding of det here and of the raster's own
 // exponent (terms up to kappa d^2 cancel to d^2); past kappa = 1e5 every block
 // is taken.
-template <int TW, int TH>
-__device__ __forceinline__ uint32_t block4_mask(float x, float y, float a, float b, float c, float op)
+template <int TW, int TH, int BW>
+__device__ __forceinline__ uint32_t block_mask(float x, float y, float a, float b, float c, float op)
 {
-    using TB = TileBlocks<TW, TH>;
-    constexpr uint32_t kAll = TB::kBlocks == 32 ? 0xffffffffu : (1u << (TB::kBlocks & 31)) - 1u;
+    constexpr int NC = TW / BW, NR = TH / 4, NB = NC * NR;
+    constexpr uint32_t kAll = NB == 32 ? 0xffffffffu : (1u << (NB & 31)) - 1u;
     if (!(op * 255.0f > 1.0f)) return 0u;      // alpha never reaches 1/255
     const float ac = a * c, det = ac - b * b;
     if (!(det > 0.0f)) return kAll;
@@ -85,19 +91,23 @@ __device__ __forceinline__ uint32_t block4_mask(float x, float y, float a, float
     const float ylo = -ey - mg, yhi = ey + mg;
     uint32_t mask = 0;
 #pragma unroll
-    for (int by = 0; by < TB::kRows; by++) {
+    for (int by = 0; by < NR; by++) {
         const float lo = fmaxf((float)(4 * by) - y, ylo), hi = fminf((float)(4 * by + 3) - y, yhi);
         const float dR = fminf(fmaxf(ys, lo), hi), dL = fminf(fmaxf(-ys, lo), hi);
         const float hR = sqrt_approx(fmaxf(0.0f, fmaf(-w * dR, dR, u)));
         const float hL = sqrt_approx(fmaxf(0.0f, fmaf(-w * dL, dL, u)));
         const float xr = x + fmaf(k, dR, hR) + mg, xl = x + fmaf(k, dL, -hL) - mg;
-        const int b0 = max(0, __float2int_ru((xl - 3.0f) * 0.25f));
-        const int b1 = min(TB::kCols - 1, __float2int_rd(xr * 0.25f));
+        const int b0 = max(0, __float2int_ru((xl - (float)(BW - 1)) * (1.0f / BW)));
+        const int b1 = min(NC - 1, __float2int_rd(xr * (1.0f / BW)));
         if (lo <= hi && b0 <= b1) {
             const uint32_t row = (2u << b1) - (1u << b0);
-            // warp-major bit order: columns 2, 3 belong to the next warp
-            const uint32_t spread = TB::kCols == 4 ? (row & 3u) | ((row & 12u) << 2) : row;
-            mask |= spread << ((by >> 1) * 4 * TB::kWarpsPerRow + (by & 1) * 2);
+            if (BW == 8) {
+                mask |= row << (by * NC);
+            } else {
+                // quads: columns 2, 3 belong to the next warp
+                const uint32_t spread = NC == 4 ? (row & 3u) | ((row & 12u) << 2) : row;
+                mask |= spread << ((by >> 1) * 2 * NC + (by & 1) * 2);
+            }
         }
     }
     return mask;

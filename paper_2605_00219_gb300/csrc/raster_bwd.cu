@@ -22,7 +22,9 @@
 // Output: one gradient record per intersection, at its emission slot, so
 // the projection backward reads each Gaussian's records contiguously.  The
 // result is deterministic (no atomics, fixed summation order).
-#include "gs_internal.cuh"
+#include <type_traits>
+
+#include "raster_blocks.cuh"
 
 namespace gs {
 
@@ -292,6 +294,429 @@ __global__ void __launch_bounds__(kBwdThreads) k_raster_bwd(Views V, const uint3
     }
 }
 
+// ===========================================================================
+// The same backward with one pixel's sums per lane replaced by groups of 8 or 16
+// lanes that walk 8x4-pixel blocks, two or four pixels per lane.
+// ===========================================================================
+
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Sums nine values over the GL = 8 or 16 lanes of a group in halving steps, in
+// the order of bfly9: (16 lanes: rows y, y + 1 first), then columns c, c + 4, then
+// c, c + 2 and c, c + 1.  Afterwards lane s of the group holds sum
+// group_sum_index<GL>(s) in `p` (-1: none); with 8 lanes, lane 0 also sum 2 in `q`.
+template <int GL>
+__device__ __forceinline__ void group_sums(const float* v, int lane, float& p, float& q)
+{
+    auto sx = [](float x, int o) { return __shfl_xor_sync(0xffffffffu, x, o); };
+    constexpr int A = GL / 2, B = GL / 4, C = GL / 8;
+    const bool ha = lane & A, hb = lane & B, hc = lane & C;
+    const float2 k01 = add2(f2(ha ? v[5] : v[0], ha ? v[6] : v[1]), f2(sx(ha ? v[0] : v[5], A), sx(ha ? v[1] : v[6], A)));
+    const float2 k23 = add2(f2(ha ? v[7] : v[2], ha ? v[8] : v[3]), f2(sx(ha ? v[2] : v[7], A), sx(ha ? v[3] : v[8], A)));
+    const float k4 = v[4] + sx(v[4], A);
+    const float2 m01 = add2(f2(hb ? k23.y : k01.x, hb ? k4 : k01.y), f2(sx(hb ? k01.x : k23.y, B), sx(hb ? k01.y : k4, B)));
+    const float m2 = k23.x + sx(k23.x, B);
+    p = (hc ? m01.y : m01.x) + sx(hc ? m01.x : m01.y, C);
+    q = m2 + sx(m2, C);
+    if (GL == 8) {
+        if ((lane & 7) == 7) p = q;
+    } else {
+        const bool hd = lane & 1;
+        p = (hd ? q : p) + sx(hd ? p : q, 1);
+    }
+}
+
+template <int GL>
+__device__ __forceinline__ int group_sum_index(int lane)
+{
+    const bool ha = lane & (GL / 2), hb = lane & (GL / 4), hc = lane & (GL / 8);
+    if (GL == 16 && (lane & 1)) return hb || hc ? -1 : ha ? 7 : 2;
+    if (hb && hc) return ha ? (GL == 8 ? 7 : -1) : 4;      // sum 4 is in both halves
+    const int k = hb ? 3 : hc ? 1 : 0;
+    return ha ? 5 + k : k;
+}
+
+// Walk of 8x4-pixel blocks of a TW x TH tile, GL lanes to a block (32 / GL pixels
+// each).  Every (entry, block) visit sums its nine values over the block's lanes
+// into a shared-memory slot of its own; an entry's slots are consecutive (a prefix
+// sum over the batch of how many blocks each entry's mask holds), and after the
+// batch one thread per entry adds them in block order.  A batch with more visits
+// than slots is walked in passes.  The sums take the order of k_raster_bwd_px at one
+// pixel per thread (rows y, y + 2; y, y + 1; columns c, c + 4; ...; blocks in
+// order), so the records are the same bits: for needle-shaped Gaussians the
+// projection backward amplifies a last-ulp change of a record up to 1e4-fold.
+//
+// Issue-bound (73% of issue slots at 20 warps per SM; ALU 55%, FMA 34%, LSU 28%;
+// 3M Gaussians, one 1080p view).  k_raster_bwd_px spends a warp visit per entry and
+// 8x4 block (2.45 an entry) with a quarter of the lanes blending; here a warp
+// iteration serves four (GL = 8: 0.68 an entry) or two (GL = 16: 1.16) visits, and
+// the packed operations both pixels of a pair.  The walk without clamps and guards
+// (no entry of the batch near alpha 0.99, everything finite) saves 26 of about 215
+// instructions: 2.80 -> 2.66 ms.
+//   GL = 8 (64 entries a batch, 10 blocks of 64 threads per SM): 1.17 -> 0.69 ms
+//     (3M, one 1080p view, FP32), 4.67 -> 2.66 ms (four views), 0.174 -> 0.100 ms
+//     (200k, 720p).  9 / 11 blocks per SM 2.72 / 2.72 ms.
+//   GL = 16 (128 entries a batch, 128 threads): 27.1 -> 20.7 us (2,000 Gaussians,
+//     128x128), 209 -> 183 us (400k, 640x360); 64 entries a batch 23.4 / 214 us.
+//     GL = 8 takes 29.0 / 242 us there: too few blocks to hide one block's chain.
+template <int TW, int TH, int GL>
+struct BwdBlocks {
+    static constexpr int kCols = TW / 8, kBlocks = kCols * (TH / 4);
+    static constexpr int kThreads = GL * kBlocks;
+    static constexpr int kGroups = 32 / GL;                   // blocks per warp
+    static constexpr int kBatch = GL == 8 ? 64 : 128;         // list entries per staged batch
+    static constexpr int kSlots = GL == 8 ? 224 : 384;        // (entry, block) sums of one pass over a batch
+    static constexpr int kBlocksPerSM = (GL == 8 ? 10 : 5) * 256 / (TW * TH);
+};
+
+template <int TW, int TH, int GL>
+__global__ void __launch_bounds__(BwdBlocks<TW, TH, GL>::kThreads, BwdBlocks<TW, TH, GL>::kBlocksPerSM)
+k_raster_bwd_blocks(Views V, const uint32_t* __restrict__ order, const uint2* __restrict__ ranges,
+                    const uint32_t* __restrict__ vals_sorted, const uint32_t* __restrict__ pid_sorted,
+                    const ProjRec* __restrict__ rec, const float* __restrict__ tfinal, const float* __restrict__ bg,
+                    const float* __restrict__ dl, const uint32_t* __restrict__ nlast, GradRec* __restrict__ gradrec,
+                    uint32_t* __restrict__ status, uint32_t cap)
+{
+    using B = BwdBlocks<TW, TH, GL>;
+    constexpr int NT = B::kThreads, NC = B::kCols, NB = B::kBlocks, BB = B::kBatch, S = B::kSlots;
+    constexpr int NG = B::kGroups;
+    constexpr int H = 16 / GL;                   // packed pixel pairs per lane
+    constexpr int IPT = (BB + NT - 1) / NT;      // staged entries per thread
+    constexpr int kEnt = 48;                     // bytes of a staged entry
+    static_assert(BB % 32 == 0 && NB <= S && 36 * (S + NB) < 65536 && kEnt * BB < 65536, "offsets fit 16 bits");
+    // staged entry: (mean x, y (tile-relative), exponent A, B), (exponent C,
+    // opacity, blue, blue), (red, red, green, green) -- the colours as pairs for
+    // the packed operations; entry BB: a stand-in that no pixel blends
+    __shared__ float4 sE[2][BB + 1][3];
+    __shared__ float sQ[2][3][BB];           // conic a, b, c
+    __shared__ uint32_t sM[2][BB], sBase[2][BB], sSlot[2][BB];
+    // slots of each run of 32 entries; bit 31: an entry's alpha may reach the
+    // 0.99 clamp, or a colour or gradient is not finite
+    __shared__ uint32_t sTot[2][BB / 32];
+    __shared__ uint32_t slist[NB][BB + 2];   // entry's byte offset | slot's byte offset << 16
+    __shared__ float part[S + NB][9];        // the last NB slots take the stand-in's sums
+    __shared__ int smax[NB];
+
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, grp = lane / GL, blk = NG * w + grp;
+    const int64_t gt = order[blockIdx.x];   // longest lists first
+    const int v = view_of_tile(V, gt);
+    const ViewDesc& vd = V.v[v];
+    const int lt = (int)(gt - vd.tile_base);
+    const int ox = (lt % vd.TX) * TW, oy = (lt / vd.TX) * TH;
+    // this lane's column and first row; its pixels are the block's four rows
+    // (8 lanes) or rows y and y + 2 (16 lanes)
+    const int px = ox + (blk % NC) * 8 + (lane & 7);
+    const int py = oy + (blk / NC) * 4 + (GL == 8 ? 0 : (lane >> 3) & 1);
+    constexpr int RS = GL == 8 ? 1 : 2;          // row step between the lane's pixels
+    const uint2 r = range_at(ranges, gt, cap, status);
+    const float fx = (float)(px - ox) + 0.5f, fy = (float)(py - oy) + 0.5f;
+    if (tid < 6) sE[tid / 3][BB][tid % 3] = make_float4(0.f, 0.f, 0.f, 0.f);
+
+    // The lane's pixels as packed pairs: rows (0, 1) and (2, 3), or (y, y + 2).
+    // Per pixel:
+    // last blended entry, compensated T after it, dL/dC, and nU = -sum_c dL/dC_c S_c
+    // with S_c the colour still to come behind an entry (from T_final bg_c):
+    // dL/dalpha = T dL/dC . col + nU / (1 - alpha)
+    const float2 one = f2(1.0f, 1.0f), zero = f2(0.f, 0.f);
+    // 1.0 the compiler cannot see through: x * one1 + y keeps the rounded x (a
+    // packed product and sum would be fused)
+    const float one1f = __uint_as_float(0x3f800000u | (cap >> 31));
+    const float2 one1 = f2(one1f, one1f);
+    float2 Th[H], Tl[H], nU[H], d0[H], d1[H], d2[H];
+    int nl[2 * H];
+    bool odd = false;            // a pixel of the tile has a non-finite dL/dC
+    {
+        float t[2 * H], e0[2 * H], e1[2 * H], e2[2 * H], u[2 * H];
+#pragma unroll
+        for (int k = 0; k < 2 * H; k++) {
+            t[k] = 1.0f; e0[k] = 0.f; e1[k] = 0.f; e2[k] = 0.f; u[k] = 0.f; nl[k] = 0;
+            if (px < vd.W && py + RS * k < vd.H) {
+                const int64_t pix = vd.pix_base + (int64_t)(py + RS * k) * vd.W + px;
+                nl[k] = (int)nlast[pix];
+                t[k] = tfinal[pix];
+                e0[k] = dl[3 * pix]; e1[k] = dl[3 * pix + 1]; e2[k] = dl[3 * pix + 2];
+                odd |= !(isfinite(e0[k]) && isfinite(e1[k]) && isfinite(e2[k]));
+                if (bg) u[k] = t[k] * fmaf(e0[k], bg[0], fmaf(e1[k], bg[1], e2[k] * bg[2]));
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < H; h++) {
+            Th[h] = f2(t[2 * h], t[2 * h + 1]);
+            Tl[h] = zero;
+            nU[h] = f2(-u[2 * h], -u[2 * h + 1]);
+            d0[h] = f2(e0[2 * h], e0[2 * h + 1]);
+            d1[h] = f2(e1[2 * h], e1[2 * h + 1]);
+            d2[h] = f2(e2[2 * h], e2[2 * h + 1]);
+        }
+        int mx = max(nl[0], nl[1]);
+        if (H == 2) mx = max(mx, max(nl[2 * H - 2], nl[2 * H - 1]));
+#pragma unroll
+        for (int o = GL / 2; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (lane % GL == 0) smax[blk] = mx;
+    }
+    odd = __syncthreads_or(odd);
+    int L = 0;
+#pragma unroll
+    for (int i = 0; i < NB; i++) L = max(L, smax[i]);
+    L = min(L, (int)(r.y - r.x));
+
+    // Batches from the back, double-buffered: the records of the batch below
+    // are copied into the other buffer while this batch is walked, and turned
+    // into staged entries in place by the thread that copied them before the
+    // barrier that ends the walk.  An entry's mask keeps the blocks it can
+    // contribute to and one of whose pixels blended at or past it; its slots
+    // follow those of the entries behind it.
+    uint32_t pid_next[IPT], e_next[IPT];
+    auto fetch = [&](int b, int buf) {     // records of batch b (pid_next), indices of the one below
+#pragma unroll
+        for (int u = 0; u < IPT; u++) {
+            const int i = tid + u * NT;
+            if (i < BB && b + i < L) {
+                rec_copy_async(sE[buf][i], rec, pid_next[u], V.pairs, status);
+                e_next[u] = vals_sorted[r.x + b + i];
+            }
+            if (i < BB && b >= BB) pid_next[u] = pid_sorted[r.x + b - BB + i];
+        }
+    };
+    auto stage = [&](int b, int buf) {
+        copy_async_wait();
+#pragma unroll
+        for (int u = 0; u < IPT; u++) {
+            const int i = tid + u * NT;
+            if (i < BB) {            // whole warps
+                uint32_t m = 0;
+                bool flag = false;
+                if (b + i < L) {
+                    const float4 qa = sE[buf][i][0], qb = sE[buf][i][1], qc = sE[buf][i][2];
+                    sE[buf][i][0] = pair_coefs(tile_mean(qa.x, qc.z, ox), tile_mean(qa.y, qc.w, oy), qa.z, qa.w, qb.x);
+                    sE[buf][i][1] = make_float4(pair_c2(qb.x), qb.y, qc.x, qc.x);
+                    sE[buf][i][2] = make_float4(qb.z, qb.z, qb.w, qb.w);
+                    // o <= 0.98 and a conic conditioned well enough that the
+                    // exponent stays below 1e-6: o 2^p < 0.99 at every pixel
+                    const float ac = qa.z * qb.x;
+                    flag = odd || !(qb.y <= 0.98f) || !(ac < 1e4f * (ac - qa.w * qa.w)) ||
+                           !(isfinite(qb.z) && isfinite(qb.w) && isfinite(qc.x));
+                    sQ[buf][0][i] = qa.z;
+                    sQ[buf][1][i] = qa.w;
+                    sQ[buf][2][i] = qb.x;
+                    sSlot[buf][i] = e_next[u];
+#pragma unroll
+                    for (int k = 0; k < NB; k++) m |= b + i < smax[k] ? 1u << k : 0u;
+                    m &= block_mask<TW, TH, 8>(qa.x - ((float)ox + 0.5f), qa.y - ((float)oy + 0.5f), qa.z, qa.w, qb.x,
+                                               qb.y);
+                }
+                sM[buf][i] = m;
+                const uint32_t c = __popc(m);
+                uint32_t x = c;             // inclusive sum over this and the higher lanes
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_down_sync(0xffffffffu, x, o);
+                    if (lane + o < 32) x += y;
+                }
+                sBase[buf][i] = x - c;
+                flag = __any_sync(0xffffffffu, flag);
+                if (lane == 0) sTot[buf][i >> 5] = x | (flag ? 0x80000000u : 0u);
+            }
+        }
+    };
+    int bb = ((L + BB - 1) / BB - 1) * BB;
+    if (bb >= 0) {
+#pragma unroll
+        for (int u = 0; u < IPT; u++) {
+            const int i = tid + u * NT;
+            pid_next[u] = i < BB && bb + i < L ? pid_sorted[r.x + bb + i] : 0u;
+        }
+        fetch(bb, 0);
+        stage(bb, 0);
+        if (bb > 0) fetch(bb - BB, 1);
+    }
+    __syncthreads();
+    const int vi = group_sum_index<GL>(lane);
+    char* const pbase = reinterpret_cast<char*>(part) + 4 * vi;
+    for (int cur = 0; bb >= 0; cur ^= 1) {
+        const int cnt = min(BB, L - bb);
+        uint32_t total = 0, flags = 0;
+#pragma unroll
+        for (int c = 0; c < BB / 32; c++) {
+            total += sTot[cur][c] & 0x7fffffffu;
+            flags |= sTot[cur][c] >> 31;
+        }
+        // last blended entries relative to the batch, as staged byte offsets
+        int nb[2 * H];
+#pragma unroll
+        for (int k = 0; k < 2 * H; k++) nb[k] = kEnt * max(-1, min(nl[k] - bb, BB));
+        const char* __restrict__ cE = reinterpret_cast<const char*>(sE[cur]);
+        // passes of at most S slots (nearly always one)
+        for (uint32_t first = 0;;) {
+            uint32_t next = total;
+            int ng[NG];
+#pragma unroll
+            for (int g = 0; g < NG; g++) ng[g] = 0;
+            uint32_t above = 0;      // slots of the higher 32-entry runs
+            if (total - first > (uint32_t)S) next = first;
+#pragma unroll
+            for (int c = BB / 32 - 1; c >= 0; c--) {
+                const int i = 32 * c + lane;
+                const uint32_t m0 = sM[cur][i], base = above + sBase[cur][i], end = base + __popc(m0);
+                const bool in = base >= first && end <= first + S;
+                const uint32_t m = in ? m0 : 0u;
+                if (in) next = max(next, end);
+                above += sTot[cur][c] & 0x7fffffffu;
+                const uint32_t q = m >> (NG * w);
+                const uint32_t s0 = base - first + __popc(m & ((1u << (NG * w)) - 1u));
+#pragma unroll
+                for (int g = 0; g < NG; g++) {
+                    const uint32_t bal = __ballot_sync(0xffffffffu, q & (1u << g));
+                    if (q & (1u << g))
+                        slist[NG * w + g][ng[g] + __popc(bal & (0xfffffffeu << lane))] =
+                            (uint32_t)(kEnt * i) | (36u * (s0 + __popc(q & ((1u << g) - 1u)))) << 16;
+                    ng[g] += __popc(bal);
+                }
+            }
+            if (total - first > (uint32_t)S) next = __reduce_max_sync(0xffffffffu, next);
+            int n = ng[0], nmax = ng[0];
+#pragma unroll
+            for (int g = 1; g < NG; g++) {
+                n = grp == g ? ng[g] : n;
+                nmax = max(nmax, ng[g]);
+            }
+            uint32_t* lp = slist[blk];
+            for (int i = n + lane % GL; i <= nmax; i += GL) lp[i] = (uint32_t)(kEnt * BB) | (36u * (S + blk)) << 16;
+            __syncwarp();
+            // (without a flag alpha needs no clamp and every product is finite)
+            auto walk = [&](auto careful_t) {
+            constexpr bool careful = decltype(careful_t)::value;
+            uint32_t ent = lp[0];
+#pragma unroll 1
+            for (int i = 0; i < nmax; i++) {
+                const uint32_t off = ent & 0xffffu, so = ent >> 16;
+                ent = lp[i + 1];
+                const float4* __restrict__ e = reinterpret_cast<const float4*>(cE + off);
+                const float4 a = e[0];
+                const float4 b = e[1];
+                const float4 rg = e[2];
+                const float dx = pix_offset(fx, a.x);
+                const PowX px2 = pair_power2_x(dx, a.z, a.w);   // shared by the lane's pixels
+                const float2 dx2 = f2(dx, dx);
+                float2 g9[9];         // sums over the lane's pairs
+#pragma unroll
+                for (int h = 0; h < H; h++) {
+                    const float2 dy = f2(pix_offset(fy + (float)(2 * h), a.y), pix_offset(fy + (float)(2 * h + RS), a.y));
+                    const float p0 = pair_power2_y(px2, dy.x, b.x), p1 = pair_power2_y(px2, dy.y, b.x);
+                    float2 G = f2(ex2_approx(p0), ex2_approx(p1));
+                    float2 as = f2(__fmul_rn(b.y, G.x), __fmul_rn(b.y, G.y));
+                    const bool h0 = (int)off < nb[2 * h] && p0 >= kPow2Min && as.x >= kAlphaMin;
+                    const bool h1 = (int)off < nb[2 * h + 1] && p1 >= kPow2Min && as.y >= kAlphaMin;
+                    // a pixel that does not blend takes alpha = 0: T and U stay, its
+                    // sums are zero (selected, so that nothing non-finite gets in)
+                    G = f2(h0 ? G.x : 0.f, h1 ? G.y : 0.f);
+                    as = f2(h0 ? as.x : 0.f, h1 ? as.y : 0.f);
+                    float2 al = as;
+                    if constexpr (careful) al = f2(fminf(kAlphaMax, as.x), fminf(kAlphaMax, as.y));
+                    // compensated T before this entry (div_one_minus on both pixels;
+                    // nom = -(1 - alpha), ne = -om_err)
+                    const float2 nom = sub2(al, one);
+                    const float2 ne = sub2(al, add2(nom, one));
+                    const float2 rc = f2(rcp_approx(-nom.x), rcp_approx(-nom.y));
+                    const float2 q = mul2(Th[h], rc);
+                    Tl[h] = mul2(fma2(q, ne, add2(fma2(q, nom, Th[h]), Tl[h])), rc);
+                    Th[h] = q;
+                    const float2 wgt = mul2(al, q);
+                    const float2 dcol =
+                        fma2(d0[h], f2(rg.x, rg.y), fma2(d1[h], f2(rg.z, rg.w), mul2(d2[h], f2(b.z, b.w))));
+                    float2 da = fma2(q, dcol, mul2(nU[h], rc));
+                    if (h0) nU[h].x = fmaf(-wgt.x, dcol.x, nU[h].x);
+                    if (h1) nU[h].y = fmaf(-wgt.y, dcol.y, nU[h].y);
+                    float2 t6 = mul2(wgt, d0[h]), t7 = mul2(wgt, d1[h]), t8 = mul2(wgt, d2[h]);
+                    if constexpr (careful) {
+                        // no gradient where the 0.99 clamp holds
+                        da = f2(h0 && as.x <= kAlphaMax ? da.x : 0.f, h1 && as.y <= kAlphaMax ? da.y : 0.f);
+                        t6 = f2(h0 ? t6.x : 0.f, h1 ? t6.y : 0.f);
+                        t7 = f2(h0 ? t7.x : 0.f, h1 ? t7.y : 0.f);
+                        t8 = f2(h0 ? t8.x : 0.f, h1 ? t8.y : 0.f);
+                    }
+                    // moments of dp = dL/dpower; the conic and the constant factors
+                    // are applied per entry
+                    const float2 dp = mul2(da, as);
+                    float2 t[9];
+                    t[0] = mul2(dp, dx2);
+                    t[1] = mul2(dy, dp);
+                    t[2] = mul2(dx2, t[0]);
+                    t[3] = mul2(dx2, t[1]);
+                    t[4] = mul2(dy, t[1]);
+                    t[5] = mul2(da, G);
+                    t[6] = t6;
+                    t[7] = t7;
+                    t[8] = t8;
+#pragma unroll
+                    for (int k = 0; k < 9; k++) g9[k] = h ? fma2(t[k], one1, g9[k]) : t[k];
+                }
+                float g[9];
+#pragma unroll
+                for (int k = 0; k < 9; k++) g[k] = __fadd_rn(g9[k].x, g9[k].y);
+                float p, q2;
+                group_sums<GL>(g, lane, p, q2);
+                if (GL == 8 || vi >= 0) *reinterpret_cast<float*>(pbase + so) = p;
+                if (GL == 8 && (lane & 7) == 0) *reinterpret_cast<float*>(pbase + so + 8) = q2;
+            }
+            };
+            if (flags) walk(std::true_type{});
+            else walk(std::false_type{});
+            const bool more = next < total;
+            if (!more && bb > 0) stage(bb - BB, cur ^ 1);
+            __syncthreads();
+            // one thread per entry adds its slots in block order and writes the
+            // record: slots 0-4 hold sums of dp (dx, dy, dx^2, dx dy, dy^2):
+            // dL/dmean = conic (sum dx dp, sum dy dp) and dL/dconic =
+            // -(sum dx^2 dp / 2, sum dx dy dp, sum dy^2 dp / 2)
+#pragma unroll
+            for (int u = 0; u < IPT; u++) {
+                const int j = tid + u * NT;
+                if (j < cnt) {
+                    uint32_t base = sBase[cur][j];
+                    for (int c = (j >> 5) + 1; c < BB / 32; c++) base += sTot[cur][c] & 0x7fffffffu;
+                    const uint32_t nsl = __popc(sM[cur][j]);
+                    if (base >= first && base + nsl <= first + S) {
+                        float sm[9];
+#pragma unroll
+                        for (int c = 0; c < 9; c++) sm[c] = 0.f;
+                        for (uint32_t k = base - first; k < base - first + nsl; k++)
+#pragma unroll
+                            for (int c = 0; c < 9; c++) sm[c] += part[k][c];
+                        const float ca = sQ[cur][0][j], cb = sQ[cur][1][j], cc = sQ[cur][2][j];
+                        const uint32_t e = sSlot[cur][j];
+                        if (GS_DCHECK(e < cap, status)) {
+                            float4* o = reinterpret_cast<float4*>(gradrec + e);
+                            o[0] = make_float4(fmaf(ca, sm[0], cb * sm[1]), fmaf(cb, sm[0], cc * sm[1]),
+                                               -0.5f * sm[2], -sm[3]);
+                            o[1] = make_float4(-0.5f * sm[4], sm[5], sm[6], sm[7]);
+                            reinterpret_cast<float*>(o + 2)[0] = sm[8];
+                        }
+                    }
+                }
+            }
+            first = next;
+            if (!more) break;
+            __syncthreads();
+        }
+        bb -= BB;
+        if (bb > 0) fetch(bb - BB, cur);   // this batch's entries are not read any more
+        __syncthreads();
+    }
+    // entries past every pixel's last blended pair receive zero gradients
+    for (uint32_t k = r.x + (uint32_t)L + tid; k < r.y; k += NT) {
+        GradRec o;
+        o.a = o.b = o.c = make_float4(0.f, 0.f, 0.f, 0.f);
+        const uint32_t e = vals_sorted[k];
+        if (GS_DCHECK(e < cap, status)) gradrec[e] = o;
+    }
+}
+
 void launch_raster_bwd_px(const Plan& P, const WsPtrs& w, const float* bg, const float* dl, cudaStream_t st);
 
 void launch_raster_bwd(const Plan& P, const WsPtrs& w, const float* image, const float* dl, cudaStream_t st)
@@ -329,8 +754,10 @@ void launch_raster_bwd(const Plan& P, const WsPtrs& w, const float* image, const
 // Second implementation: pixels across threads, per-Gaussian gradients
 // reduced across each warp's pixels by shuffles (no atomics).
 //
-// One CTA per tile, one thread per pixel, each warp an 8x4 pixel block (so a
-// small Gaussian touches few warps).  Every pixel walks its own list prefix
+// One CTA per tile, one, two or four pixels per thread, each warp an 8x4, 8x8 or
+// 8x16 pixel block (so a small Gaussian touches few warps).  This form now runs
+// for 8x8 tiles, for two pixels per thread with FP32 moments and for four; the
+// others walk blocks by lane groups (k_raster_bwd_blocks, below).  Every pixel walks its own list prefix
 // back to front from its last blended entry: T before an entry is recovered
 // by a compensated division of T after it by (1 - alpha) (div_one_minus:
 // hardware reciprocal, exact remainder, carried low part), and the colour
@@ -631,19 +1058,34 @@ void launch_raster_bwd_px(const Plan& P, const WsPtrs& w, const float* bg, const
     k_raster_bwd_px<BS, TW, PPT><<<grid, BS, 0, st>>>(V, w.tile_order, w.ranges, w.vals_sorted, w.pid_sorted, \
                                                       w.rec, w.tfinal, bg, dl, w.nlast, w.gradrec, &w.hdr->status,   \
                                                       (uint32_t)P.cap)
+#define GS_RBB(TW, TH, GL)                                                                                    \
+    k_raster_bwd_blocks<TW, TH, GL><<<grid, BwdBlocks<TW, TH, GL>::kThreads, 0, st>>>(                         \
+        V, w.tile_order, w.ranges, w.vals_sorted, w.pid_sorted, w.rec, w.tfinal, bg, dl, w.nlast, w.gradrec,   \
+        &w.hdr->status, (uint32_t)P.cap)
+    // 16-wide tiles with one pixel per thread (the default) walk 8x4 blocks,
+    // and so do two pixels per thread with BF16 moments: their stored rounding
+    // (4e-3) hides the other summation order, which FP32 moments keep.  Four
+    // visits per warp (GL = 8) need two waves of resident blocks to hide a
+    // tile's chain: 2,040 tiles 98.9 us against 83.1 us for GL = 16, 3,600 tiles
+    // 100 / 114 us (200k) and 252 / 223 us (1M, sparser), 5,700 tiles 252 / 294 us.
+    const bool blocks = ppt == 1 || (ppt == 2 && P.mom_bf16);
+    const bool full = V.tiles >= 2 * (int64_t)P.sm_count * BwdBlocks<16, 16, 8>::kBlocksPerSM * 256 / (V.tw * V.th);
     if (V.tw == 8) {
         if (ppt == 1) GS_RBP(64, 8, 1);
         else GS_RBP(32, 8, 2);
     } else if (V.th == 16) {
-        if (ppt == 1) GS_RBP(256, 16, 1);
+        if (blocks && full) GS_RBB(16, 16, 8);
+        else if (blocks) GS_RBB(16, 16, 16);
         else if (ppt == 2) GS_RBP(128, 16, 2);
         else GS_RBP(64, 16, 4);
     } else {
-        if (ppt == 1) GS_RBP(512, 16, 1);
+        if (blocks && full) GS_RBB(16, 32, 8);
+        else if (blocks) GS_RBB(16, 32, 16);
         else if (ppt == 2) GS_RBP(256, 16, 2);
         else GS_RBP(128, 16, 4);
     }
 #undef GS_RBP
+#undef GS_RBB
 }
 
 }  // namespace gs

@@ -70,7 +70,7 @@ k_raster_fwd(Views V, const uint32_t* __restrict__ order, const uint2* __restric
         sE[buf][i][0] = pair_coefs(tile_mean(qa.x, qc.z, ox), tile_mean(qa.y, qc.w, oy), qa.z, qa.w, qb.x);
         sE[buf][i][1] = make_float4(pair_c2(qb.x), qb.y, qb.z, qb.w);
         sE[buf][i][2].x = qc.x;
-        sM[buf][i] = block4_mask<TW, TH>(qa.x - ((float)ox + 0.5f), qa.y - ((float)oy + 0.5f), qa.z, qa.w, qb.x, qb.y);
+        sM[buf][i] = block_mask<TW, TH, 4>(qa.x - ((float)ox + 0.5f), qa.y - ((float)oy + 0.5f), qa.z, qa.w, qb.x, qb.y);
     };
     // chunk 0 is staged directly; afterwards the records of chunk i + 1 are
     // copied to shared memory while chunk i is composited (the pair indices
