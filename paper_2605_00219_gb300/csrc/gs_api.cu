@@ -143,7 +143,7 @@ static bool plan_build(Plan& P, const int64_t* scene_n, int32_t n_scenes, const 
     P.count_scan_parts = (pairs + kScanBlock - 1) / kScanBlock;
     P.tile_scan_parts = (tiles + kScanBlock - 1) / kScanBlock;
     P.raster_blocks = tiles;
-    const int64_t loss_blocks = std::max<int64_t>((3 * pixels + 2047) / 2048, 2 * ssim_tiles(V));
+    const int64_t loss_blocks = std::max<int64_t>((3 * pixels + 2047) / 2048, 2 * ssim_blocks(V));
 
     size_t o = 0;
     auto take = [&](size_t bytes) {

@@ -8,24 +8,74 @@
 // With the window moments mu_x, mu_y, E[x^2], E[y^2], E[xy] at q,
 //   dSSIM_sum / dx_p = (w * A)(p) + 2 x_p (w * B)(p) + y_p (w * Cc)(p),
 // A = dSSIM/dmu_x, B = dSSIM/dE[x^2], Cc = dSSIM/dE[xy] at each q (the window
-// is symmetric).  One CTA per 16x16 tile of a view: x and y are staged with a
-// 10-pixel halo, separable 11-tap passes give the five moments at the 26x26
-// positions whose windows reach the tile, then A, B, Cc there, and two more
-// separable passes give the gradient at the tile's pixels -- one kernel, no
+// is symmetric).  One CTA per 32x31 tile of a view and colour channel: x and y are
+// staged with a 10-pixel halo, separable 11-tap passes give the five moments at
+// the 42x41 positions whose windows reach the tile, then A, B, Cc there, and two
+// more separable passes give the gradient at the tile's pixels -- one kernel, no
 // intermediate image in global memory, no layout conversion.
+//
+// Issue- and FP32-bound (68% of issue slots, 2.8 IPC at 24 warps per SM; 53% of the
+// LSU): about 400 FP32 operations a pixel and channel with the halos, 8 x 22 of
+// them the windows' own.  Every pass is register-blocked along its window: a thread
+// reads the 11 + n - 1 values of n neighbouring outputs once (n = 9, 7, 6, 4 for the
+// four passes) instead of 11 values an output, and the tile height 31 gives each
+// pass just under 256 tasks, one per thread (51 rows x 5 groups, 42 columns x 6 groups,
+// 41 rows x 6 groups, 32 columns x 8 groups).  Moments and partials are packed pairs
+// (FFMA2).  The three channels of a tile are neighbouring CTAs, so that small images
+// fill the chip and the channels' accesses to one pixel meet in L2.
+// Four 1080p views: 1.43 -> 0.56 ms against one output a thread in 16x16 tiles;
+// 403x301: 33 -> 16 us.  With the staging loads four rows at a time 0.74 ms (one
+// round trip of all 13 rows 0.56).
 //
 // The moments are taken about a per-tile shift (x and y at the tile's centre
 // pixel): variances and the covariance are shift-invariant, and with values
 // near the local mean E[x^2] - mu_x^2 no longer cancels in FP32 on flat
 // image regions.  Zero padding becomes padding with -shift.
-#include "gs_internal.cuh"
+#include "raster_blocks.cuh"
 
 namespace gs {
 
-constexpr int kSsT = 16;                 // output tile
-constexpr int kSsR = 5;                  // window radius
-constexpr int kSsQ = kSsT + 2 * kSsR;    // 26: positions whose window reaches the tile
-constexpr int kSsX = kSsT + 4 * kSsR;    // 36: staged pixels per side
+constexpr int kSsR = 5;                    // window radius
+constexpr int kSsW = 32, kSsH = 31;        // output tile
+constexpr int kQw = kSsW + 2 * kSsR;       // 42 x 41: positions whose window reaches the tile
+constexpr int kQh = kSsH + 2 * kSsR;
+constexpr int kXw = kSsW + 4 * kSsR;       // 52 x 51: staged pixels
+constexpr int kXh = kSsH + 4 * kSsR;
+// outputs per thread of the four passes, and their tasks
+constexpr int kN1 = 9, kN2 = 7, kN3 = 6, kN4 = 4;
+constexpr int kG1 = (kQw + kN1 - 1) / kN1, kG2 = (kQh + kN2 - 1) / kN2;
+constexpr int kG3 = (kSsW + kN3 - 1) / kN3, kG4 = (kSsH + kN4 - 1) / kN4;
+constexpr int kSsThreads = 256;
+static_assert(kXh * kG1 <= kSsThreads && kQw * kG2 <= kSsThreads && kQh * kG3 <= kSsThreads &&
+                  kSsW * kG4 <= kSsThreads, "one task per thread in every pass");
+// shared-memory pitches: odd in the unit read across rows (no bank conflicts),
+// with room for the outputs past the edge that a last group computes and drops
+constexpr int kPx = kG1 * kN1 + 2 * kSsR;          // 55 float2
+constexpr int kPm = 43;                            // float4 / float
+constexpr int kPa = 47;                            // float2 / float (46 read)
+constexpr int kPh = 33;                            // float2 / float
+constexpr int kRm = kG2 * kN2 + 2 * kSsR;          // 52 rows
+constexpr int kRh = kG4 * kN4 + 2 * kSsR;          // 42 rows
+static_assert(kPa >= kG3 * kN3 + 2 * kSsR, "abc columns");
+struct SsimSmem {
+    union {
+        float2 xy[kXh][kPx];               // (x, y) about the shift
+        struct {
+            float2 ab[kQh][kPa];           // (A, B)
+            float c[kQh][kPa];             // Cc
+        } abc;
+    };
+    union {
+        struct {
+            float4 m03[kRm][kPm];          // (mu_x, mu_y, E[x^2], E[y^2]) of the rows
+            float m4[kRm][kPm];            // E[xy]
+        } h;
+        struct {
+            float2 ab[kRh][kPh];
+            float c[kRh][kPh];
+        } habc;
+    };
+};
 constexpr float kSsC1 = 0.01f * 0.01f;
 
 // Window tap k (0..10): exp(-(k - 5)^2 / (2 * 1.5^2)) normalised to unit sum,
@@ -46,7 +96,7 @@ __device__ __forceinline__ int ssim_view_of_tile(const Views& V, int64_t t, int6
 {
     int64_t base = 0;
     for (int v = 0; v < V.n; v++) {
-        const int64_t nt = (int64_t)((V.v[v].W + kSsT - 1) / kSsT) * ((V.v[v].H + kSsT - 1) / kSsT);
+        const int64_t nt = (int64_t)((V.v[v].W + kSsW - 1) / kSsW) * ((V.v[v].H + kSsH - 1) / kSsH);
         if (t < base + nt || v == V.n - 1) {
             first = base;
             return v;
@@ -72,142 +122,220 @@ __device__ __forceinline__ float pix_mask(uchar4 t)
 }
 
 template <bool MASK>
-__global__ void __launch_bounds__(256) k_loss_l1_ssim(Views V, const float* __restrict__ image,
-                                                      const uchar4* __restrict__ target, float lam,
-                                                      float inv_n, float* __restrict__ dl,
-                                                      float* __restrict__ part, WsHeader* __restrict__ hdr)
+__global__ void __launch_bounds__(kSsThreads, 3) k_loss_l1_ssim(Views V, const float* __restrict__ image,
+                                                                const uchar4* __restrict__ target, float lam,
+                                                                float inv_n, float* __restrict__ dl,
+                                                                float* __restrict__ part, WsHeader* __restrict__ hdr)
 {
-    __shared__ float2 sxy[kSsX][kSsX + 1];   // (x, y) about the shift
-    // moments and partials interleaved, so each tap of the next pass reads
-    // them with vector loads: (mu_x, mu_y, E[x^2], E[y^2]), E[xy]; (A, B), Cc
-    __shared__ float4 hm03[kSsX][kSsQ];
-    __shared__ float hm4[kSsX][kSsQ];
-    __shared__ float2 abc01[kSsQ][kSsQ];
-    __shared__ float abc2[kSsQ][kSsQ + 1];
-    __shared__ float2 habc01[kSsQ][kSsT];
-    __shared__ float habc2[kSsQ][kSsT];
-    __shared__ float red[2][8];
+    extern __shared__ __align__(16) unsigned char ssim_smem[];
+    SsimSmem& sm = *reinterpret_cast<SsimSmem*>(ssim_smem);
+    __shared__ float red[2][kSsThreads / 32];
     __shared__ bool is_last;
 
     const int tid = threadIdx.x;
     int64_t first;
-    const int v = ssim_view_of_tile(V, blockIdx.x, first);
+    const int c = (int)(blockIdx.x % 3u);        // colour channel
+    const int64_t tile = blockIdx.x / 3u;
+    const int v = ssim_view_of_tile(V, tile, first);
     const ViewDesc& vd = V.v[v];
-    const int lt = (int)(blockIdx.x - first);
-    const int TX = (vd.W + kSsT - 1) / kSsT;
-    const int ox = (lt % TX) * kSsT, oy = (lt / TX) * kSsT;
-    const int pc = tid % kSsT, pr = tid / kSsT;
-    const int px = ox + pc, py = oy + pr;
-    const bool pin = px < vd.W && py < vd.H;
-    const int64_t ppix = vd.pix_base + (int64_t)py * vd.W + px;
-    float l1 = 0.f, ss = 0.f;
+    const int lt = (int)(tile - first);
+    const int TX = (vd.W + kSsW - 1) / kSsW;
+    const int ox = (lt % TX) * kSsW, oy = (lt / TX) * kSsH;
+    float l1 = 0.f, ss = 0.f, shx, shy;
 
-    const int64_t cpix = vd.pix_base + (int64_t)min(oy + kSsT / 2, vd.H - 1) * vd.W + min(ox + kSsT / 2, vd.W - 1);
-    for (int c = 0; c < 3; c++) {
-        const uchar4 tc = target[cpix];
+    const int64_t cpix = vd.pix_base + (int64_t)min(oy + kSsH / 2, vd.H - 1) * vd.W + min(ox + kSsW / 2, vd.W - 1);
+    const uchar4 tc = target[cpix];
+    const float ic = image[3 * cpix + c];
+    // 64 threads a row (52 used), so that no index is divided; all loads of a
+    // thread are in flight together, with the shift's (one memory round trip a tile)
+    {
+        constexpr int RS = kSsThreads / 64, NR = (kXh + RS - 1) / RS;
+        const int col = tid & 63, r0 = tid >> 6, x = ox - 2 * kSsR + col;
+        const bool xin = col < kXw && x >= 0 && x < vd.W;
+        const int64_t pix0 = vd.pix_base + (int64_t)(oy - 2 * kSsR + r0) * vd.W + x;
+        float xi[NR];
+        uchar4 ti[NR];
+#pragma unroll
+        for (int k = 0; k < NR; k++) {
+            const int r = r0 + RS * k, y = oy - 2 * kSsR + r;
+            xi[k] = 0.f;
+            ti[k] = make_uchar4(0, 0, 0, 0);
+            if (xin && r < kXh && y >= 0 && y < vd.H) {
+                const int64_t pix = pix0 + (int64_t)(RS * k) * vd.W;
+                xi[k] = image[3 * pix + c];
+                ti[k] = target[pix];
+            }
+        }
         const float mc = pix_mask<MASK>(tc);
-        const float shx = image[3 * cpix + c] * mc, shy = target_channel(tc, c) * mc;
-        __syncthreads();
-        for (int i = tid; i < kSsX * kSsX; i += 256) {
-            const int r = i / kSsX, col = i % kSsX;
-            const int x = ox - 2 * kSsR + col, y = oy - 2 * kSsR + r;
-            float a = 0.f, b = 0.f;
-            if (x >= 0 && y >= 0 && x < vd.W && y < vd.H) {
-                const int64_t pix = vd.pix_base + (int64_t)y * vd.W + x;
-                const uchar4 t4 = target[pix];
-                const float m = pix_mask<MASK>(t4);
-                a = image[3 * pix + c] * m;
-                b = target_channel(t4, c) * m;
-            }
-            sxy[r][col] = make_float2(a - shx, b - shy);
-        }
-        __syncthreads();
-        // horizontal pass: 5 moments at 36 rows x 26 columns
-        for (int i = tid; i < kSsX * kSsQ; i += 256) {
-            const int r = i / kSsQ, q = i % kSsQ;
-            float m0 = 0.f, m1 = 0.f, m2 = 0.f, m3 = 0.f, m4 = 0.f;
+        // (a non-finite centre pixel shifts by nothing: it reaches only its own windows)
+        shx = isfinite(ic * mc) ? ic * mc : 0.f;
+        shy = target_channel(tc, c) * mc;
 #pragma unroll
-            for (int k = 0; k <= 2 * kSsR; k++) {
-                const float w = ssim_w(k);
-                const float2 xy = sxy[r][q + k];
-                const float a = xy.x, b = xy.y;
-                m0 = fmaf(w, a, m0);
-                m1 = fmaf(w, b, m1);
-                m2 = fmaf(w, a * a, m2);
-                m3 = fmaf(w, b * b, m3);
-                m4 = fmaf(w, a * b, m4);
-            }
-            hm03[r][q] = make_float4(m0, m1, m2, m3);
-            hm4[r][q] = m4;
+        for (int k = 0; k < NR; k++) {
+            const int r = r0 + RS * k;
+            const float m = pix_mask<MASK>(ti[k]);
+            if (col < kXw && r < kXh) sm.xy[r][col] = make_float2(xi[k] * m - shx, target_channel(ti[k], c) * m - shy);
         }
-        __syncthreads();
-        // vertical pass, SSIM and its partials at 26 x 26 positions
-        for (int i = tid; i < kSsQ * kSsQ; i += 256) {
-            const int qr = i / kSsQ, qc = i % kSsQ;
-            float m[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    }
+    __syncthreads();
+    // horizontal pass: 5 moments at 51 rows x 42 columns
+    if (tid < kXh * kG1) {
+        const int r = tid % kXh, q0 = (tid / kXh) * kN1;
+        float2 m01[kN1], m23[kN1];
+        float m4[kN1];
 #pragma unroll
-            for (int k = 0; k <= 2 * kSsR; k++) {
-                const float w = ssim_w(k);
-                const float4 a = hm03[qr + k][qc];
-                m[0] = fmaf(w, a.x, m[0]);
-                m[1] = fmaf(w, a.y, m[1]);
-                m[2] = fmaf(w, a.z, m[2]);
-                m[3] = fmaf(w, a.w, m[3]);
-                m[4] = fmaf(w, hm4[qr + k][qc], m[4]);
+        for (int o = 0; o < kN1; o++) {
+            m01[o] = m23[o] = make_float2(0.f, 0.f);
+            m4[o] = 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < kN1 + 2 * kSsR; j++) {
+            const float2 xy = sm.xy[r][q0 + j];
+            const float2 sq = mul2(xy, xy);
+            const float pr = xy.x * xy.y;
+#pragma unroll
+            for (int o = 0; o < kN1; o++) {
+                if (j - o < 0 || j - o > 2 * kSsR) continue;
+                const float w = ssim_w(j - o);
+                m01[o] = fma2(f2(w, w), xy, m01[o]);
+                m23[o] = fma2(f2(w, w), sq, m23[o]);
+                m4[o] = fmaf(w, pr, m4[o]);
             }
-            const int x = ox - kSsR + qc, y = oy - kSsR + qr;
+        }
+#pragma unroll
+        for (int o = 0; o < kN1; o++)
+            if (q0 + o < kQw) {
+                sm.h.m03[r][q0 + o] = make_float4(m01[o].x, m01[o].y, m23[o].x, m23[o].y);
+                sm.h.m4[r][q0 + o] = m4[o];
+            }
+    }
+    __syncthreads();
+    // vertical pass, SSIM and its partials at 42 columns x 41 rows
+    if (tid < kQw * kG2) {
+        const int qc = tid % kQw, r0 = (tid / kQw) * kN2;
+        float2 m01[kN2], m23[kN2];
+        float m4[kN2];
+#pragma unroll
+        for (int o = 0; o < kN2; o++) {
+            m01[o] = m23[o] = make_float2(0.f, 0.f);
+            m4[o] = 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < kN2 + 2 * kSsR; j++) {
+            const float4 a = sm.h.m03[r0 + j][qc];
+            const float e = sm.h.m4[r0 + j][qc];
+#pragma unroll
+            for (int o = 0; o < kN2; o++) {
+                if (j - o < 0 || j - o > 2 * kSsR) continue;
+                const float w = ssim_w(j - o);
+                m01[o] = fma2(f2(w, w), f2(a.x, a.y), m01[o]);
+                m23[o] = fma2(f2(w, w), f2(a.z, a.w), m23[o]);
+                m4[o] = fmaf(w, e, m4[o]);
+            }
+        }
+        const int x = ox - kSsR + qc;
+#pragma unroll
+        for (int o = 0; o < kN2; o++) {
+            const int qr = r0 + o, y = oy - kSsR + qr;
+            if (qr >= kQh) break;
             float A = 0.f, B = 0.f, Cc = 0.f;
             if (x >= 0 && y >= 0 && x < vd.W && y < vd.H) {
-                const float mx = m[0] + shx, my = m[1] + shy;
-                const float vx = m[2] - m[0] * m[0], vy = m[3] - m[1] * m[1], cxy = m[4] - m[0] * m[1];
+                const float mx = m01[o].x + shx, my = m01[o].y + shy;
+                const float vx = m23[o].x - m01[o].x * m01[o].x, vy = m23[o].y - m01[o].y * m01[o].y;
+                const float cxy = m4[o] - m01[o].x * m01[o].y;
                 const float a1 = 2.f * mx * my + kSsC1, a2 = 2.f * cxy + kSsC2;
                 const float b1 = mx * mx + my * my + kSsC1, b2 = vx + vy + kSsC2;
-                const float ib = 1.0f / (b1 * b2);
-                const float s = a1 * a2 * ib;
-                A = 2.f * my * (a2 - a1) * ib - 2.f * mx * s / b1 + 2.f * mx * s / b2;
-                B = -s / b2;
+                // one hardware reciprocal (an ulp): 1 / b1 = b2 ib, 1 / b2 = b1 ib
+                const float ib = __fdividef(1.0f, b1 * b2);
+                const float s = a1 * a2 * ib, ib2 = b1 * ib;
+                A = 2.f * (my * (a2 - a1) * ib + mx * s * (ib2 - b2 * ib));
+                B = -s * ib2;
                 Cc = 2.f * a1 * ib;
-                if (qr >= kSsR && qr < kSsR + kSsT && qc >= kSsR && qc < kSsR + kSsT) ss += s;
+                if (qr >= kSsR && qr < kSsR + kSsH && qc >= kSsR && qc < kSsR + kSsW) ss += s;
             }
-            abc01[qr][qc] = make_float2(A, B);
-            abc2[qr][qc] = Cc;
+            sm.abc.ab[qr][qc] = make_float2(A, B);
+            sm.abc.c[qr][qc] = Cc;
         }
-        __syncthreads();
-        // horizontal pass of A, B, Cc: 26 rows x 16 columns
-        for (int i = tid; i < kSsQ * kSsT; i += 256) {
-            const int r = i / kSsT, q = i % kSsT;
-            float a = 0.f, b = 0.f, d = 0.f;
+    }
+    __syncthreads();
+    // the tile's own pixels, requested before the last two passes need them
+    const int pc = tid % kSsW, pr0 = (tid / kSsW) * kN4, px = ox + pc;
+    float ox4[kN4];
+    uchar4 ot4[kN4];
 #pragma unroll
-            for (int k = 0; k <= 2 * kSsR; k++) {
-                const float w = ssim_w(k);
-                const float2 ab = abc01[r][q + k];
-                a = fmaf(w, ab.x, a);
-                b = fmaf(w, ab.y, b);
-                d = fmaf(w, abc2[r][q + k], d);
+    for (int o = 0; o < kN4; o++) {
+        const int py = oy + pr0 + o;
+        ox4[o] = 0.f;
+        ot4[o] = make_uchar4(0, 0, 0, 0);
+        if (pr0 + o < kSsH && px < vd.W && py < vd.H) {
+            const int64_t ppix = vd.pix_base + (int64_t)py * vd.W + px;
+            ox4[o] = image[3 * ppix + c];
+            ot4[o] = target[ppix];
+        }
+    }
+    // horizontal pass of A, B, Cc: 41 rows x 32 columns
+    if (tid < kQh * kG3) {
+        const int r = tid % kQh, q0 = (tid / kQh) * kN3;
+        float2 ab[kN3];
+        float d[kN3];
+#pragma unroll
+        for (int o = 0; o < kN3; o++) {
+            ab[o] = make_float2(0.f, 0.f);
+            d[o] = 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < kN3 + 2 * kSsR; j++) {
+            const float2 a = sm.abc.ab[r][q0 + j];
+            const float e = sm.abc.c[r][q0 + j];
+#pragma unroll
+            for (int o = 0; o < kN3; o++) {
+                if (j - o < 0 || j - o > 2 * kSsR) continue;
+                const float w = ssim_w(j - o);
+                ab[o] = fma2(f2(w, w), a, ab[o]);
+                d[o] = fmaf(w, e, d[o]);
             }
-            habc01[r][q] = make_float2(a, b);
-            habc2[r][q] = d;
         }
-        __syncthreads();
-        // vertical pass at the tile's pixel; combine with the L1 term
-        float wa = 0.f, wb = 0.f, wc = 0.f;
 #pragma unroll
-        for (int k = 0; k <= 2 * kSsR; k++) {
-            const float w = ssim_w(k);
-            const float2 ab = habc01[pr + k][pc];
-            wa = fmaf(w, ab.x, wa);
-            wb = fmaf(w, ab.y, wb);
-            wc = fmaf(w, habc2[pr + k][pc], wc);
+        for (int o = 0; o < kN3; o++)
+            if (q0 + o < kSsW) {
+                sm.habc.ab[r][q0 + o] = ab[o];
+                sm.habc.c[r][q0 + o] = d[o];
+            }
+    }
+    __syncthreads();
+    // vertical pass at the tile's pixels; combine with the L1 term
+    if (tid < kSsW * kG4) {
+        float2 ab[kN4];
+        float d[kN4];
+#pragma unroll
+        for (int o = 0; o < kN4; o++) {
+            ab[o] = make_float2(0.f, 0.f);
+            d[o] = 0.f;
         }
-        if (pin) {
-            const uchar4 t4 = target[ppix];
-            const float m = pix_mask<MASK>(t4);
-            const float x = image[3 * ppix + c] * m, y = target_channel(t4, c) * m;
-            const float d = x - y;
-            const float dS = wa + 2.f * x * wb + y * wc;
-            const float sg = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
+#pragma unroll
+        for (int j = 0; j < kN4 + 2 * kSsR; j++) {
+            const float2 a = sm.habc.ab[pr0 + j][pc];
+            const float e = sm.habc.c[pr0 + j][pc];
+#pragma unroll
+            for (int o = 0; o < kN4; o++) {
+                if (j - o < 0 || j - o > 2 * kSsR) continue;
+                const float w = ssim_w(j - o);
+                ab[o] = fma2(f2(w, w), a, ab[o]);
+                d[o] = fmaf(w, e, d[o]);
+            }
+        }
+#pragma unroll
+        for (int o = 0; o < kN4; o++) {
+            const int py = oy + pr0 + o;
+            if (pr0 + o >= kSsH || px >= vd.W || py >= vd.H) continue;
+            const int64_t ppix = vd.pix_base + (int64_t)py * vd.W + px;
+            const float m = pix_mask<MASK>(ot4[o]);
+            const float x = ox4[o] * m, y = target_channel(ot4[o], c) * m;
+            const float df = x - y;
+            const float dS = ab[o].x + 2.f * x * ab[o].y + y * d[o];
+            const float sg = df > 0.f ? 1.f : (df < 0.f ? -1.f : 0.f);
             dl[3 * ppix + c] = MASK ? m * (((1.f - lam) * sg - lam * dS) * inv_n) : ((1.f - lam) * sg - lam * dS) * inv_n;
-            l1 += fabsf(d);
+            l1 += fabsf(df);
         }
     }
     // per-CTA partial sums (L1, SSIM), then the last CTA adds them in order
@@ -251,23 +379,29 @@ __global__ void __launch_bounds__(256) k_loss_l1_ssim(Views V, const float* __re
     }
 }
 
-int64_t ssim_tiles(const Views& V)
+int64_t ssim_blocks(const Views& V)
 {
     int64_t t = 0;
-    for (int v = 0; v < V.n; v++) t += (int64_t)((V.v[v].W + kSsT - 1) / kSsT) * ((V.v[v].H + kSsT - 1) / kSsT);
-    return t;
+    for (int v = 0; v < V.n; v++) t += (int64_t)((V.v[v].W + kSsW - 1) / kSsW) * ((V.v[v].H + kSsH - 1) / kSsH);
+    return 3 * t;
 }
 
 void launch_loss_l1_ssim(const Plan& P, const WsPtrs& w, const float* image, const void* target_rgba8, float lam,
                          bool alpha_mask, float* dl, cudaStream_t st)
 {
-    const int64_t tiles = ssim_tiles(P.views);
+    const int64_t blocks = ssim_blocks(P.views);
     const float inv_n = 1.0f / (float)(3 * P.views.pixels);
     const uchar4* t = static_cast<const uchar4*>(target_rgba8);
-    if (alpha_mask)
-        k_loss_l1_ssim<true><<<(unsigned)tiles, 256, 0, st>>>(P.views, image, t, lam, inv_n, dl, w.loss_part, w.hdr);
-    else
-        k_loss_l1_ssim<false><<<(unsigned)tiles, 256, 0, st>>>(P.views, image, t, lam, inv_n, dl, w.loss_part, w.hdr);
+#define GS_SSIM(MASK)                                                                                               \
+    do {                                                                                                            \
+        cudaFuncSetAttribute(k_loss_l1_ssim<MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize,                     \
+                             (int)sizeof(SsimSmem));                                                                \
+        k_loss_l1_ssim<MASK><<<(unsigned)blocks, kSsThreads, sizeof(SsimSmem), st>>>(P.views, image, t, lam, inv_n, \
+                                                                                    dl, w.loss_part, w.hdr);       \
+    } while (0)
+    if (alpha_mask) GS_SSIM(true);
+    else GS_SSIM(false);
+#undef GS_SSIM
 }
 
 }  // namespace gs
