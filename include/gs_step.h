@@ -312,7 +312,7 @@ const char* gs_status_str(gs_status s);
  * *loss = sum |image - target| / n_values written to the DEVICE float `loss`.
  * All four pointers are device memory owned by the caller.
  *
- * Its scratch (block partial sums and a completion counter, about 128 KiB)
+ * Its scratch (block partial sums and a completion counter, about 5 KiB)
  * is a static array inside the library, held by every GPU that loads the
  * library until the process exits.  The first call on a device looks up that
  * array's device address (with the device current) and caches it; make that
