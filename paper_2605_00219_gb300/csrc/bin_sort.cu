@@ -50,33 +50,6 @@ void launch_fill_u32(uint32_t* p, int64_t n, uint32_t value, cudaStream_t st)
 // Exclusive scan of u32 (reduce, scan of block sums, down-sweep)
 // ---------------------------------------------------------------------------
 
-template <int T>
-__device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* warp_sums, uint32_t* total)
-{
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) warp_sums[w] = x;
-    __syncthreads();
-    if (w == 0) {
-        uint32_t s = lane < T / 32 ? warp_sums[lane] : 0u;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
-        }
-        if (lane < T / 32) warp_sums[lane] = s;
-    }
-    __syncthreads();
-    uint32_t before = w > 0 ? warp_sums[w - 1] : 0u;
-    if (total) *total = warp_sums[T / 32 - 1];
-    return before + x - v;
-}
-
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t* __restrict__ in,
                                                                const uint32_t* __restrict__ in2, int64_t n,
                                                                uint32_t* __restrict__ part)
@@ -207,11 +180,6 @@ static void scan_tile_counts(const Plan& P, const WsPtrs& w, cudaStream_t st)
     const int64_t tiles = P.views.tiles;
     scan_launch(w.tile_cnt, w.tile_cnt + tiles, w.tile_cur, tiles, w.scan_part, w.hdr, nullptr, 0u, w.ranges,
                 w.tile_cnt + tiles, st);
-}
-
-void scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* part, cudaStream_t st)
-{
-    scan_launch(in, nullptr, out, n, part, nullptr, nullptr, 0u, nullptr, nullptr, st);
 }
 
 // ---------------------------------------------------------------------------

@@ -154,6 +154,35 @@ __device__ __forceinline__ int view_of_tile(const Views& V, int64_t t)
     return v;
 }
 
+// Exclusive scan of one value per thread over a block of T threads (warp_sums:
+// shared, 32 words); *total the block's sum.
+template <int T>
+__device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* warp_sums, uint32_t* total)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_sums[w] = x;
+    __syncthreads();
+    if (w == 0) {
+        uint32_t s = lane < T / 32 ? warp_sums[lane] : 0u;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += y;
+        }
+        if (lane < T / 32) warp_sums[lane] = s;
+    }
+    __syncthreads();
+    uint32_t before = w > 0 ? warp_sums[w - 1] : 0u;
+    if (total) *total = warp_sums[T / 32 - 1];
+    return before + x - v;
+}
+
 // --------------------------------------------------------------------------
 // FP32 binning, bit-specified: every operation is one correctly rounded
 // binary32 operation in the written order (explicit _rn intrinsics, which the
