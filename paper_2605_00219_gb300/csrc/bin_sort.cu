@@ -7,16 +7,16 @@
 // as a bucketing by tile followed by a sort of each tile's short list.
 //
 //   index offset : exclusive scan of the per-pair tile counts, in
-//                  Gaussian-major pair order (reduce-then-scan, three
-//                  launches, no inter-block waiting): a Gaussian's
-//                  intersections in all views are consecutive emission slots
+//                  Gaussian-major pair order: a Gaussian's intersections in all
+//                  views are consecutive emission slots.  Sums per 1,024 pairs,
+//                  one block scans them, and the emission scans its pairs (no
+//                  inter-block waiting, no second pass over the counts)
 //   tile ranges  : the projection's traversal already counted the entries of
 //                  every tile; their exclusive scan gives each tile's
 //                  [start, end) in the sorted arrays and its scatter cursor
-//   generate keys: second scan-line pass; each intersection takes the next
-//                  slot of its tile (an atomic cursor) and stores its depth
-//                  code and emission slot there, and its pair at the
-//                  emission slot
+//   generate keys: from the tile spans the projection kept, each intersection
+//                  goes to its rank's or the next free place of its tile (depth
+//                  code and emission slot), and its pair to the emission slot
 //   sorting      : one thread block per tile sorts the tile's entries by
 //                  (depth code, emission slot) -- unique, so the arrival
 //                  order of the atomics does not matter -- and writes the
@@ -47,144 +47,296 @@ void launch_fill_u32(uint32_t* p, int64_t n, uint32_t value, cudaStream_t st)
 }
 
 // ---------------------------------------------------------------------------
-// Exclusive scan of u32 (reduce, scan of block sums, down-sweep)
+// Emission slots, tile ranges and launch order
 // ---------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t* __restrict__ in,
-                                                               const uint32_t* __restrict__ in2, int64_t n,
-                                                               uint32_t* __restrict__ part)
+// Launch order of the raster kernels and the tile sort: tiles by decreasing list
+// length, bucketed by floor(log2(length + 1)).  Blocks are dispatched roughly in
+// index order, so the longest tiles start first and the short ones fill the
+// tail (longest-processing-time scheduling).  Within a bucket the order
+// follows shared-memory atomics; it decides only when a tile runs, never its
+// result.
+__device__ __forceinline__ int len_bucket(uint32_t len) { return 31 - __clz(len + 1u); }
+
+// The sort's size classes are runs of buckets: long >= 2047 entries (buckets
+// 11+), medium 1023-2046 (10), short 255-1022 (8, 9), tiny <= 254 (0-7).  One
+// thread: the class sizes, and each bucket's first place in the order (in place).
+__device__ __forceinline__ void order_places(uint32_t* cnt, WsHeader* hdr)
 {
-    __shared__ uint32_t ws[32];
-    const int64_t base = (int64_t)blockIdx.x * kScanBlock;
-    uint32_t s = 0;
-#pragma unroll
-    for (int i = 0; i < kScanItems; i++) {
-        int64_t idx = base + i * kScanThreads + threadIdx.x;
-        if (idx < n) s += in[idx] + (in2 ? in2[idx] : 0u);
+    uint32_t cls[4] = {0u, 0u, 0u, 0u};
+    uint32_t run = 0;
+    for (int b = 31; b >= 0; b--) {
+        const uint32_t c = cnt[b];
+        cls[b >= 11 ? 0 : b == 10 ? 1 : b >= 8 ? 2 : 3] += c;
+        cnt[b] = run;
+        run += c;
     }
-    uint32_t tot;
-    block_excl_scan<kScanThreads>(s, ws, &tot);
-    if (threadIdx.x == 0) part[blockIdx.x] = tot;
+    for (int c = 0; c < 4; c++) hdr->sort_class[c] = cls[c];
 }
 
-// Single block: exclusive scan of the block sums in place; grand total at
-// part[nparts].  With total_at (the scan of the pair counts; hdr then not
-// null): the total is K, also written to total_at (the offsets' last entry),
-// and the capacity check sets k_eff = K when it fits, else 0 (nothing is
-// emitted) with GS_STATUS_CAPACITY.
-__global__ void __launch_bounds__(1024) k_scan_part(uint32_t* __restrict__ part, int64_t nparts,
-                                                    WsHeader* __restrict__ hdr, uint32_t* __restrict__ total_at,
-                                                    uint32_t cap)
+// Intersections of one group of kPairGroup pairs, summed by one warp.
+__device__ __forceinline__ uint32_t pair_group_sum(const uint32_t* __restrict__ count, int64_t pairs, int64_t group)
 {
-    __shared__ uint32_t ws[32];
+    // (every load of the group in flight at once)
+    uint32_t c[kPairGroup / 32], s = 0;
+#pragma unroll
+    for (int k = 0; k < kPairGroup / 32; k++) {
+        const int64_t q = group * kPairGroup + 32 * k + (threadIdx.x & 31);
+        c[k] = q < pairs ? count[q] : 0u;
+    }
+#pragma unroll
+    for (int k = 0; k < kPairGroup / 32; k++) s += c[k];
+    return __reduce_add_sync(0xffffffffu, s);
+}
+
+// Exclusive scan in place of the pair groups' intersection counts by one block of
+// 1,024 threads (each warp one run of them: sums, then prefixes), K, the
+// offsets' last entry and the capacity check: k_eff = K when it fits, else 0
+// (nothing is emitted) with GS_STATUS_CAPACITY.  Returns whether K fits.
+__device__ bool scan_gpart(uint32_t* __restrict__ gpart, int64_t blocks, WsHeader* __restrict__ hdr,
+                           uint32_t* __restrict__ total_at, uint32_t cap, unsigned long long* ws)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t per = ((blocks + 31) / 32 + 31) & ~(int64_t)31;       // whole warp accesses
+    const int64_t b0 = min(per * w, blocks), b1 = min(b0 + per, blocks);
+    unsigned long long sum = 0;
+#pragma unroll 4
+    for (int64_t i = b0 + lane; i < b1; i += 32) sum += gpart[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) ws[w] = sum;
+    __syncthreads();
+    unsigned long long before = 0, total = 0;
+    for (int k = 0; k < 32; k++) {
+        if (k < w) before += ws[k];
+        total += ws[k];
+    }
+    uint32_t carry = (uint32_t)before;
+#pragma unroll 4
+    for (int64_t i0 = b0; i0 < b1; i0 += 32) {
+        const uint32_t v = i0 + lane < b1 ? gpart[i0 + lane] : 0u;
+        uint32_t x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (i0 + lane < b1) gpart[i0 + lane] = carry + x - v;
+        carry += __shfl_sync(0xffffffffu, x, 31);
+    }
+    const bool fits = total <= cap;
+    if (threadIdx.x == 0) {
+        hdr->k_required = total;
+        hdr->k_eff = fits ? (uint32_t)total : 0u;
+        if (!fits) atomicOr(&hdr->status, GS_STATUS_CAPACITY);
+        *total_at = (uint32_t)total;
+    }
+    return fits;
+}
+
+// Range of a tile: its list, empty when the tile is or when K exceeds the capacity.
+__device__ __forceinline__ uint2 tile_range(uint32_t start, uint32_t len, bool fits)
+{
+    return fits && len ? make_uint2(start, start + len) : make_uint2(0u, 0u);
+}
+
+// Up to kScanBlock tiles, one block: emission-slot scan, K, and for every tile
+// its start (exclusive scan of both counters), range, the cursor of the other
+// pairs' entries (start + the ranked entries, written over their counter) and its
+// place in the launch order.  Latency-bound; seven launches of the same work took
+// 25 us at 64 tiles and 36 us at 3,600 (8 us here, and 4 us of k_sort_sums).
+__global__ void __launch_bounds__(1024) k_sort_setup(const uint32_t* __restrict__ count, int64_t pairs, bool summed,
+                                                     uint32_t* gpart, int64_t gblocks, int tiles,
+                                                     uint32_t* cnt, uint32_t* __restrict__ tile_cur,
+                                                     uint2* __restrict__ ranges, uint32_t* __restrict__ order,
+                                                     uint32_t* __restrict__ total_at, WsHeader* __restrict__ hdr,
+                                                     uint32_t cap)
+{
+    constexpr int IT = kScanBlock / 1024;
+    __shared__ unsigned long long ws64[32];
+    __shared__ uint32_t ws[32], hist[32];
+    __shared__ uint32_t buf[kScanBlock];
+    if (threadIdx.x < 32) hist[threadIdx.x] = 0;
+    uint32_t c0[IT], len[IT];
+#pragma unroll
+    for (int k = 0; k < IT; k++) {
+        const int t = k * 1024 + threadIdx.x;
+        c0[k] = t < tiles ? cnt[t] : 0u;
+        len[k] = t < tiles ? c0[k] + cnt[tiles + t] : 0u;
+        buf[t] = len[k];
+    }
+    if (!summed) {
+        for (int64_t g = threadIdx.x >> 5; g < gblocks; g += 32) {
+            const uint32_t t = pair_group_sum(count, pairs, g);
+            if ((threadIdx.x & 31) == 0) gpart[g] = t;
+        }
+        __syncthreads();
+    }
+    const bool fits = scan_gpart(gpart, gblocks, hdr, total_at, cap, ws64);     // (synchronises)
+    uint32_t own[IT], s = 0;
+#pragma unroll
+    for (int k = 0; k < IT; k++) {
+        own[k] = s;
+        s += buf[threadIdx.x * IT + k];
+    }
+    const uint32_t ex = block_excl_scan<1024>(s, ws, nullptr);
+#pragma unroll
+    for (int k = 0; k < IT; k++) buf[threadIdx.x * IT + k] = ex + own[k];
+#pragma unroll
+    for (int k = 0; k < IT; k++)
+        if (k * 1024 + (int)threadIdx.x < tiles) atomicAdd(&hist[len_bucket(fits ? len[k] : 0u)], 1u);
+    __syncthreads();
+    if (threadIdx.x == 0) order_places(hist, hdr);
+#pragma unroll
+    for (int k = 0; k < IT; k++) {
+        const int t = k * 1024 + threadIdx.x;
+        if (t < tiles) {
+            const uint32_t s0 = buf[t];
+            tile_cur[t] = s0;
+            ranges[t] = tile_range(s0, len[k], fits);
+            cnt[tiles + t] = s0 + c0[k];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < IT; k++) {
+        const int t = k * 1024 + threadIdx.x;
+        if (t < tiles) order[atomicAdd(&hist[len_bucket(fits ? len[k] : 0u)], 1u)] = (uint32_t)t;
+    }
+}
+
+// More pairs or tiles: sums first.  Blocks below gblocks16: the sums of 16 pair
+// groups, one per warp; the others (more than kScanBlock tiles, the same work in
+// three launches): sum and list-length histogram of kScanBlock tiles per block
+// (part: [blocks] sums, then [blocks][32] buckets);
+__global__ void __launch_bounds__(kScanThreads) k_sort_sums(const uint32_t* __restrict__ count, int64_t pairs,
+                                                            uint32_t* __restrict__ gpart, int64_t gblocks,
+                                                            unsigned gblocks16, int64_t tiles,
+                                                            const uint32_t* __restrict__ cnt,
+                                                            uint32_t* __restrict__ part)
+{
+    __shared__ uint32_t ws[32], hist[32];
+    if (blockIdx.x < gblocks16) {
+        const int64_t g = (int64_t)blockIdx.x * (kScanThreads / 32) + (threadIdx.x >> 5);
+        if (g < gblocks) {
+            const uint32_t t = pair_group_sum(count, pairs, g);
+            if ((threadIdx.x & 31) == 0) gpart[g] = t;
+        }
+        return;
+    }
+    const int64_t blk = blockIdx.x - gblocks16, blocks = gridDim.x - gblocks16;
+    if (threadIdx.x < 32) hist[threadIdx.x] = 0;
+    __syncthreads();
+    uint32_t s = 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; k++) {
+        const int64_t t = blk * kScanBlock + k * kScanThreads + threadIdx.x;
+        if (t < tiles) {
+            const uint32_t len = cnt[t] + cnt[tiles + t];
+            s += len;
+            atomicAdd(&hist[len_bucket(len)], 1u);
+        }
+    }
+    uint32_t tot;
+    block_excl_scan<kScanThreads>(s, ws, &tot);      // (synchronises)
+    if (threadIdx.x == 0) part[blk] = tot;
+    if (threadIdx.x < 32) part[blocks + 32 * blk + threadIdx.x] = hist[threadIdx.x];
+}
+
+// one block: the emission-slot scan and K, the blocks' tile starts, and each
+// (block, bucket)'s first place in the order (when K exceeds the capacity every
+// list is empty: all tiles in bucket 0);
+__global__ void __launch_bounds__(1024) k_sort_parts(uint32_t* __restrict__ gpart, int64_t gblocks, int64_t tiles,
+                                                     uint32_t* __restrict__ part, int64_t nparts,
+                                                     uint32_t* __restrict__ total_at, WsHeader* __restrict__ hdr,
+                                                     uint32_t cap)
+{
+    __shared__ unsigned long long ws64[32];
+    __shared__ uint32_t ws[32], place[32];
+    const bool fits = scan_gpart(gpart, gblocks, hdr, total_at, cap, ws64);
     uint32_t carry = 0;
     for (int64_t b = 0; b < nparts; b += 1024) {
-        int64_t i = b + threadIdx.x;
-        uint32_t v = i < nparts ? part[i] : 0u;
+        const int64_t i = b + threadIdx.x;
+        const uint32_t v = i < nparts ? part[i] : 0u;
         uint32_t tot;
-        uint32_t ex = block_excl_scan<1024>(v, ws, &tot);
+        const uint32_t ex = block_excl_scan<1024>(v, ws, &tot);
         if (i < nparts) part[i] = carry + ex;
         carry += tot;
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        part[nparts] = carry;
-        if (total_at) {
-            hdr->k_required = carry;
-            hdr->k_eff = carry <= cap ? carry : 0u;
-            if (carry > cap) atomicOr(&hdr->status, GS_STATUS_CAPACITY);
-            *total_at = carry;
+    uint32_t* hist = part + nparts;
+    const int b = threadIdx.x & 31;
+    if (threadIdx.x < 32) {
+        uint32_t c = 0;
+        for (int64_t i = 0; i < nparts; i++) {
+            if (!fits) hist[32 * i + b] = b ? 0u : (uint32_t)min((int64_t)kScanBlock, tiles - i * kScanBlock);
+            c += hist[32 * i + b];
+        }
+        place[b] = c;
+        __syncwarp();
+        if (threadIdx.x == 0) order_places(place, hdr);
+        __syncwarp();
+        uint32_t run = place[b];
+        for (int64_t i = 0; i < nparts; i++) {
+            const uint32_t h = hist[32 * i + b];
+            hist[32 * i + b] = run;
+            run += h;
         }
     }
 }
 
-// Down-sweep: out[i] = exclusive prefix of in[i] (+ in2[i]).  With ranges
-// (the scan of the tile counters, in = entries of ranked pairs, in2 = the
-// others' entries; hdr then not null, its K already set): also each tile's
-// range [start, start + both counts) --
-// [0, 0) when empty, and every range empty when K exceeds the capacity --
-// and the cursor for the other pairs' entries, start + the ranked entries,
-// written over in2 (cur2, the same array).
-__global__ void __launch_bounds__(kScanThreads) k_scan_down(const uint32_t* in, const uint32_t* in2, int64_t n,
-                                                             const uint32_t* __restrict__ part, uint32_t* out,
-                                                             uint2* __restrict__ ranges, uint32_t* cur2,
-                                                             const WsHeader* __restrict__ hdr)
+// starts, ranges, cursors and places.
+__global__ void __launch_bounds__(kScanThreads) k_tile_down(int64_t tiles, uint32_t* cnt,
+                                                            const uint32_t* __restrict__ part,
+                                                            uint32_t* __restrict__ tile_cur,
+                                                            uint2* __restrict__ ranges, uint32_t* __restrict__ order,
+                                                            const WsHeader* __restrict__ hdr)
 {
+    __shared__ uint32_t ws[32], hist[32];
     __shared__ uint32_t buf[kScanBlock];
-    __shared__ uint32_t ws[32];
     const int64_t base = (int64_t)blockIdx.x * kScanBlock;
-    if (base >= n) return;
+    if (threadIdx.x < 32) hist[threadIdx.x] = part[gridDim.x + 32 * (int64_t)blockIdx.x + threadIdx.x];
+    const bool fits = hdr->k_eff == hdr->k_required;
+    uint32_t c0[kScanItems], len[kScanItems];
 #pragma unroll
-    for (int i = 0; i < kScanItems; i++) {
-        int64_t idx = base + i * kScanThreads + threadIdx.x;
-        buf[i * kScanThreads + threadIdx.x] = idx < n ? in[idx] + (in2 ? in2[idx] : 0u) : 0u;
+    for (int k = 0; k < kScanItems; k++) {
+        const int l = k * kScanThreads + threadIdx.x;
+        c0[k] = base + l < tiles ? cnt[base + l] : 0u;
+        len[k] = base + l < tiles ? c0[k] + cnt[tiles + base + l] : 0u;
+        buf[l] = len[k];
     }
     __syncthreads();
-    uint32_t loc[kScanItems];
-    uint32_t s = 0;
+    uint32_t own[kScanItems], s = 0;
 #pragma unroll
-    for (int i = 0; i < kScanItems; i++) {
-        loc[i] = s;
-        s += buf[threadIdx.x * kScanItems + i];
+    for (int k = 0; k < kScanItems; k++) {
+        own[k] = s;
+        s += buf[threadIdx.x * kScanItems + k];
     }
-    uint32_t ex = block_excl_scan<kScanThreads>(s, ws, nullptr) + part[blockIdx.x];
-    // (the list lengths are read back before the prefixes replace them)
-    uint32_t len[kScanItems];
-    if (ranges) {
+    const uint32_t ex = block_excl_scan<kScanThreads>(s, ws, nullptr) + part[blockIdx.x];
 #pragma unroll
-        for (int i = 0; i < kScanItems; i++) len[i] = buf[threadIdx.x * kScanItems + i];
-    }
-#pragma unroll
-    for (int i = 0; i < kScanItems; i++) buf[threadIdx.x * kScanItems + i] = ex + loc[i];
+    for (int k = 0; k < kScanItems; k++) buf[threadIdx.x * kScanItems + k] = ex + own[k];
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < kScanItems; i++) {
-        int64_t idx = base + i * kScanThreads + threadIdx.x;
-        if (idx < n) out[idx] = buf[i * kScanThreads + threadIdx.x];
-    }
-    if (ranges) {
-        const bool fits = hdr->k_eff == hdr->k_required;
-#pragma unroll
-        for (int i = 0; i < kScanItems; i++) {
-            const int64_t idx = base + threadIdx.x * kScanItems + i;
-            if (idx < n) {
-                const uint32_t s0 = ex + loc[i], c = len[i];
-                ranges[idx] = fits && c ? make_uint2(s0, s0 + c) : make_uint2(0u, 0u);
-                cur2[idx] = s0 + in[idx];
-            }
+    for (int k = 0; k < kScanItems; k++) {
+        const int l = k * kScanThreads + threadIdx.x;
+        const int64_t t = base + l;
+        if (t < tiles) {
+            const uint32_t s0 = buf[l];
+            tile_cur[t] = s0;
+            ranges[t] = tile_range(s0, len[k], fits);
+            cnt[tiles + t] = s0 + c0[k];
+            order[atomicAdd(&hist[len_bucket(fits ? len[k] : 0u)], 1u)] = (uint32_t)t;
         }
     }
-}
-
-static void scan_launch(const uint32_t* in, const uint32_t* in2, uint32_t* out, int64_t n, uint32_t* part,
-                        WsHeader* hdr, uint32_t* total_at, uint32_t cap, uint2* ranges, uint32_t* cur2,
-                        cudaStream_t st)
-{
-    const int64_t nparts = (n + kScanBlock - 1) / kScanBlock;
-    k_scan_reduce<<<(unsigned)nparts, kScanThreads, 0, st>>>(in, in2, n, part);
-    k_scan_part<<<1, 1024, 0, st>>>(part, nparts, hdr, total_at, cap);
-    k_scan_down<<<(unsigned)nparts, kScanThreads, 0, st>>>(in, in2, n, part, out, ranges, cur2, hdr);
-}
-
-// Offsets of the pair counts, K and the capacity check.
-static void scan_pair_counts(const Plan& P, const WsPtrs& w, cudaStream_t st)
-{
-    scan_launch(w.count, nullptr, w.offset, P.views.pairs, w.scan_part, w.hdr, w.offset + P.views.pairs,
-                (uint32_t)P.cap, nullptr, nullptr, st);
-}
-
-// Tile starts, ranges and the other pairs' cursors from the two tile
-// counters (after scan_pair_counts: the ranges read K and k_eff).
-static void scan_tile_counts(const Plan& P, const WsPtrs& w, cudaStream_t st)
-{
-    const int64_t tiles = P.views.tiles;
-    scan_launch(w.tile_cnt, w.tile_cnt + tiles, w.tile_cur, tiles, w.scan_part, w.hdr, nullptr, 0u, w.ranges,
-                w.tile_cnt + tiles, st);
 }
 
 // ---------------------------------------------------------------------------
 // Generate keys into tile buckets
 // ---------------------------------------------------------------------------
+
+constexpr int kEmitThreads = 256;
+// Tiles of a one- or two-band pair that its own lane places.
+constexpr uint32_t kEmitLane = 16;
 
 // One thread per Gaussian-major pair q: its intersections take emission
 // slots offset[q] + i in traversal order; each is placed in its tile's list
@@ -193,92 +345,130 @@ static void scan_tile_counts(const Plan& P, const WsPtrs& w, cudaStream_t st)
 // pair's entries go to tile start + the rank the projection took; the other
 // pairs' entries take the next free place after the ranked ones (an atomic
 // cursor per tile), and the rare pair of more than two bands repeats the
-// traversal from its binning geometry.
-__global__ void __launch_bounds__(256, 6) k_emit(Views V, const uint32_t* __restrict__ count,
-                                                 const uint32_t* __restrict__ offset, const ProjRec* __restrict__ rec,
+// traversal from its binning geometry.  A pair of more than kEmitLane tiles or
+// two bands is placed by its whole warp: one lane's serial walk of the largest
+// footprints was a third of the launch on a room of 200k Gaussians (32 -> 22 us).
+// 3M Gaussians, 4 views: 265 us with the slot scan inside, against 240 + 49 us for
+// the emission and a separate scan (5 blocks per SM; 6 / 4: 274 / 285 us).
+//
+// The pair's first emission slot is its group's scanned sum, the counts of the
+// group's earlier blocks (at most three), and a scan of the block's own counts.  It is
+// written to offset for the backward.
+__global__ void __launch_bounds__(kEmitThreads, 5) k_emit(Views V, const uint32_t* __restrict__ count,
+                                                 const uint32_t* __restrict__ gpart,
+                                                 uint32_t* __restrict__ offset, const ProjRec* __restrict__ rec,
                                                  const uint4* __restrict__ span, const uint4* __restrict__ rank,
                                                  const uint32_t* __restrict__ tile_start, uint32_t* tile_over,
                                                  uint2* __restrict__ bucket, uint32_t* __restrict__ pid,
                                                  WsHeader* __restrict__ hdr)
 {
-    const int64_t qi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (qi >= V.pairs) return;
+    __shared__ uint32_t ws[32], earlier[kEmitThreads / 32];
+    const int64_t qb = (int64_t)blockIdx.x * kEmitThreads, qi = qb + threadIdx.x;
     // the pair's loads are issued together, before any of them is tested
     // (one memory round trip instead of three); span and ranks are stale
     // for a pair without tiles and a pair that is not ranked, and unused
-    const uint32_t kreq = hdr->k_required, keff = hdr->k_eff;
-    const uint32_t cnt = count[qi];
-    const uint32_t off = offset[qi];
-    const uint4 sp = span[qi];
-    const uint4 rk4 = rank[qi];
+    const unsigned long long kreq = hdr->k_required;
+    const uint32_t keff = hdr->k_eff;
+    const bool valid = qi < V.pairs;
+    const uint32_t cnt = valid ? count[qi] : 0u;
+    uint4 sp, rk4;
+    if (valid) {
+        sp = span[qi];
+        rk4 = rank[qi];
+    }
+    uint32_t pre = 0;
+    for (int64_t q = qi - kEmitThreads; q >= qb - qb % kPairGroup; q -= kEmitThreads) pre += count[q];
+    pre = __reduce_add_sync(0xffffffffu, pre);
+    if ((threadIdx.x & 31) == 0) earlier[threadIdx.x >> 5] = pre;
+    uint32_t off = gpart[qb / kPairGroup] + block_excl_scan<kEmitThreads>(cnt, ws, nullptr);   // (synchronises)
+#pragma unroll
+    for (int k = 0; k < kEmitThreads / 32; k++) off += earlier[k];
+    if (valid) offset[qi] = off;
     if (keff != kreq) return;     // over capacity: nothing is emitted
-    if (cnt == 0) return;
     int s = 0;
     while (s + 1 < V.n_scenes && V.qbase[s + 1] <= qi) s++;
-    const int nv = V.nv[s];
-    const int64_t local = qi - V.qbase[s];
-    const int64_t g = local / nv;
-    const int v = V.view_of[s][(int)(local - g * nv)];
+    const uint32_t nv = (uint32_t)V.nv[s];
+    const uint32_t local = (uint32_t)(qi - V.qbase[s]);     // pairs < 2^31
+    const uint32_t g = local / nv;
+    const int v = cnt ? V.view_of[s][local - g * nv] : 0;
     const ViewDesc& vd = V.v[v];
-    const uint32_t p = (uint32_t)(vd.pair_base + g);
-    const uint32_t low = (sp.x & 0x7FFFFFu) >> vd.drop;
+    const uint32_t p = (uint32_t)vd.pair_base + g;
     const uint32_t nb = (sp.x >> 24) & 3u;
-    uint32_t* cur = tile_over + vd.tile_base;
-    if (nb == kSpanMany) {
-        const float4 ra = rec[p].a;
-        BinGeom gm;
-        gm.mx = ra.x; gm.my = ra.y;
-        gm.a = __uint_as_float(sp.y); gm.b = __uint_as_float(sp.z); gm.c = __uint_as_float(sp.w);
-        gm.det = FS(FM(gm.a, gm.c), FM(gm.b, gm.b));
-        gm.r2 = cull_r2(rec[p].b.y);   // same bits as in the projection pass
-        gm.mant = sp.x & 0x7FFFFFu;
-        gm.valid = 1;
-        scanline_tiles(gm, V.tw, V.th, vd.TX, vd.TY, [&](uint32_t i, uint32_t tile) {
-            const uint32_t e = off + i;
-            const uint32_t slot = atomicAdd(cur + tile, 1u);
-            if (GS_DCHECK(slot < hdr->k_eff && e < hdr->k_eff, &hdr->status)) {
-                bucket[slot] = make_uint2(low, e);
-                pid[e] = p;
-            }
-        });
-        return;
-    }
-    const bool rows = (sp.x >> 26) & 1u;
-    const uint32_t TX = (uint32_t)vd.TX;
-    const uint32_t c0 = sp.y & 0xFFFFu, c1 = sp.y >> 16;
-    if ((sp.x >> 27) & 1u) {
-        // ranked: at most kRankMax tiles, no atomics
-        const uint32_t rk[kRankMax] = {rk4.x, rk4.y, rk4.z, rk4.w};
-        const uint32_t* __restrict__ st0 = tile_start + vd.tile_base;
+    // a pair of many tiles is placed by the whole warp, below
+    const bool wide = cnt != 0 && (nb == kSpanMany || cnt > kEmitLane);
+    if (cnt != 0 && !wide) {
+        const uint32_t low = (sp.x & 0x7FFFFFu) >> vd.drop;
+        uint32_t* cur = tile_over + vd.tile_base;
+        const bool rows = (sp.x >> 26) & 1u;
+        const uint32_t TX = (uint32_t)vd.TX;
+        const uint32_t c0 = sp.y & 0xFFFFu, c1 = sp.y >> 16;
+        if ((sp.x >> 27) & 1u) {
+            // ranked: at most kRankMax tiles, no atomics
+            const uint32_t rk[kRankMax] = {rk4.x, rk4.y, rk4.z, rk4.w};
+            const uint32_t* __restrict__ st0 = tile_start + vd.tile_base;
 #pragma unroll
-        for (uint32_t u = 0; u < kRankMax; u++) {
-            const uint32_t e = off + u;
-            if (u < cnt) {
-                const uint32_t slot = st0[span_tile(u, rows, TX, c0, c1, sp.z, sp.w)] + rk[u];
-                if (GS_DCHECK(slot < hdr->k_eff && e < hdr->k_eff, &hdr->status)) {
-                    bucket[slot] = make_uint2(low, e);
-                    pid[e] = p;
+            for (uint32_t u = 0; u < kRankMax; u++) {
+                const uint32_t e = off + u;
+                if (u < cnt) {
+                    const uint32_t slot = st0[span_tile(u, rows, TX, c0, c1, sp.z, sp.w)] + rk[u];
+                    if (GS_DCHECK(slot < hdr->k_eff && e < hdr->k_eff, &hdr->status)) {
+                        bucket[slot] = make_uint2(low, e);
+                        pid[e] = p;
+                    }
+                }
+            }
+        } else {
+            // one or two bands: the cursors taken four at a time so that the
+            // atomics' round trips overlap
+            for (uint32_t i0 = 0; i0 < cnt; i0 += 4) {
+                uint32_t slot[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const uint32_t i = i0 + u;
+                    if (i < cnt) slot[u] = atomicAdd(cur + span_tile(i, rows, TX, c0, c1, sp.z, sp.w), 1u);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const uint32_t i = i0 + u, e = off + i;
+                    if (i < cnt && GS_DCHECK(slot[u] < hdr->k_eff && e < hdr->k_eff, &hdr->status)) {
+                        bucket[slot[u]] = make_uint2(low, e);
+                        pid[e] = p;
+                    }
                 }
             }
         }
-        return;
     }
-    // one or two bands: the cursors taken four at a time so that the
-    // atomics' round trips overlap
-    for (uint32_t i0 = 0; i0 < cnt; i0 += 4) {
-        uint32_t slot[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const uint32_t i = i0 + u;
-            if (i < cnt) slot[u] = atomicAdd(cur + span_tile(i, rows, TX, c0, c1, sp.z, sp.w), 1u);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const uint32_t i = i0 + u, e = off + i;
-            if (i < cnt && GS_DCHECK(slot[u] < hdr->k_eff && e < hdr->k_eff, &hdr->status)) {
-                bucket[slot[u]] = make_uint2(low, e);
-                pid[e] = p;
+    for (uint32_t m = __ballot_sync(0xffffffffu, wide); m; m &= m - 1u) {
+        const int k = __ffs(m) - 1;
+        auto from = [&](uint32_t x) { return __shfl_sync(0xffffffffu, x, k); };
+        const uint4 ks = make_uint4(from(sp.x), from(sp.y), from(sp.z), from(sp.w));
+        const uint32_t koff = from(off), kcnt = from(cnt), kp = from(p);
+        const ViewDesc& kd = V.v[from((uint32_t)v)];
+        const uint32_t low = (ks.x & 0x7FFFFFu) >> kd.drop;
+        uint32_t* cur = tile_over + kd.tile_base;
+        auto place = [&](uint32_t i, uint32_t tile) {
+            const uint32_t e = koff + i, slot = atomicAdd(cur + tile, 1u);
+            if (GS_DCHECK(slot < hdr->k_eff && e < hdr->k_eff, &hdr->status)) {
+                bucket[slot] = make_uint2(low, e);
+                pid[e] = kp;
             }
+        };
+        if (((ks.x >> 24) & 3u) == kSpanMany) {
+            // the traversal again, from the binning geometry (same bits)
+            const float4 ra = rec[kp].a;
+            BinGeom gm;
+            gm.mx = ra.x; gm.my = ra.y;
+            gm.a = __uint_as_float(ks.y); gm.b = __uint_as_float(ks.z); gm.c = __uint_as_float(ks.w);
+            gm.det = FS(FM(gm.a, gm.c), FM(gm.b, gm.b));
+            gm.r2 = cull_r2(rec[kp].b.y);
+            gm.mant = ks.x & 0x7FFFFFu;
+            gm.valid = 1;
+            uint32_t bands;
+            warp_scanline(gm, V.tw, V.th, kd.TX, kd.TY, bands, [](uint32_t, bool, int, int, int) {}, place);
+        } else {
+            const bool rows = (ks.x >> 26) & 1u;
+            for (uint32_t i = threadIdx.x & 31; i < kcnt; i += 32)
+                place(i, span_tile(i, rows, (uint32_t)kd.TX, ks.y & 0xFFFFu, ks.y >> 16, ks.z, ks.w));
         }
     }
 }
@@ -589,60 +779,37 @@ __global__ void __launch_bounds__(kTileSortSmall) k_tile_sort_short(Views V, con
     tile_sort_group(V, gt, r.x, n, sk + w * 256, g, bucket, pid, keys_sorted, vals_sorted, pid_sorted, status, cap);
 }
 
-// Launch order of the raster kernels: tiles by decreasing list length,
-// bucketed by floor(log2(length + 1)).  Blocks are dispatched roughly in
-// index order, so the longest tiles start first and the short ones fill the
-// tail (longest-processing-time scheduling).  Within a bucket the order
-// follows shared-memory atomics; it decides only when a tile runs, never its
-// result.
-__global__ void __launch_bounds__(1024) k_tile_order(int64_t tiles, const uint2* __restrict__ ranges,
-                                                     uint32_t* __restrict__ order, WsHeader* __restrict__ hdr)
-{
-    __shared__ uint32_t cnt[32];
-    if (threadIdx.x < 32) cnt[threadIdx.x] = 0;
-    __syncthreads();
-    for (int64_t t = threadIdx.x; t < tiles; t += blockDim.x) {
-        const uint2 r = ranges[t];
-        atomicAdd(&cnt[31 - __clz(r.y - r.x + 1u)], 1u);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        // the sort's size classes are runs of buckets: long >= 2047 entries
-        // (buckets 11+), medium 1023-2046 (10), short 255-1022 (8, 9), tiny
-        // <= 254 (0-7)
-        uint32_t cls[4] = {0u, 0u, 0u, 0u};
-        for (int b = 0; b < 32; b++) cls[b >= 11 ? 0 : b == 10 ? 1 : b >= 8 ? 2 : 3] += cnt[b];
-        for (int c = 0; c < 4; c++) hdr->sort_class[c] = cls[c];
-        uint32_t run = 0;
-        for (int b = 31; b >= 0; b--) {
-            const uint32_t c = cnt[b];
-            cnt[b] = run;
-            run += c;
-        }
-    }
-    __syncthreads();
-    for (int64_t t = threadIdx.x; t < tiles; t += blockDim.x) {
-        const uint2 r = ranges[t];
-        order[atomicAdd(&cnt[31 - __clz(r.y - r.x + 1u)], 1u)] = (uint32_t)t;
-    }
-}
-
 // ---------------------------------------------------------------------------
 
 void launch_bin_sort(const Plan& P, const WsPtrs& w, cudaStream_t st)
 {
     const Views& V = P.views;
     const uint32_t cap = (uint32_t)P.cap;
-    // index offset (Gaussian-major pair order), K and the capacity check
-    scan_pair_counts(P, w, st);
-    // tile starts, ranges and the other pairs' cursors from the tile counters
-    scan_tile_counts(P, w, st);
-    k_tile_order<<<1, 1024, 0, st>>>(V.tiles, w.ranges, w.tile_order, w.hdr);
+    // emission-slot scan, K and the capacity check; tile starts, ranges, the other
+    // pairs' cursors and the launch order
+    uint32_t* const total_at = w.offset + V.pairs;
+    const bool one = V.tiles <= kScanBlock;
+    const bool sums = !one || P.pair_groups > 64;      // else the one block sums the pairs itself
+    const unsigned nparts = one ? 0u : (unsigned)P.tile_scan_parts;
+    if (sums) {
+        const unsigned gb = (unsigned)((P.pair_groups + kScanThreads / 32 - 1) / (kScanThreads / 32));
+        k_sort_sums<<<gb + nparts, kScanThreads, 0, st>>>(w.count, V.pairs, w.gpart, P.pair_groups, gb, V.tiles,
+                                                          w.tile_cnt, w.tile_part);
+    }
+    if (one) {
+        k_sort_setup<<<1, 1024, 0, st>>>(w.count, V.pairs, sums, w.gpart, P.pair_groups, (int)V.tiles, w.tile_cnt,
+                                         w.tile_cur, w.ranges, w.tile_order, total_at, w.hdr, cap);
+    } else {
+        k_sort_parts<<<1, 1024, 0, st>>>(w.gpart, P.pair_groups, V.tiles, w.tile_part, nparts, total_at, w.hdr, cap);
+        k_tile_down<<<nparts, kScanThreads, 0, st>>>(V.tiles, w.tile_cnt, w.tile_part, w.tile_cur, w.ranges,
+                                                     w.tile_order, w.hdr);
+    }
     // generate keys into the tile buckets
     {
-        const int64_t blocks = (V.pairs + 255) / 256;
-        k_emit<<<(unsigned)blocks, 256, 0, st>>>(V, w.count, w.offset, w.rec, w.span, w.rank, w.tile_cur,
-                                                 w.tile_cnt + V.tiles, w.bucket, w.pid, w.hdr);
+        const int64_t blocks = (V.pairs + kEmitThreads - 1) / kEmitThreads;
+        k_emit<<<(unsigned)blocks, kEmitThreads, 0, st>>>(V, w.count, w.gpart, w.offset, w.rec, w.span, w.rank,
+                                                          w.tile_cur, w.tile_cnt + V.tiles, w.bucket, w.pid,
+                                                          w.hdr);
     }
     // sort each tile's list
     {

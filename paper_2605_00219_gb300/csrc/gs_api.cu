@@ -43,7 +43,8 @@ WsPtrs carve(const Plan& P, void* ws)
     w.nlast = reinterpret_cast<uint32_t*>(b + P.off_nlast);
     w.tfinal = reinterpret_cast<float*>(b + P.off_tfinal);
     w.gradrec = reinterpret_cast<GradRec*>(b + P.off_gradrec);
-    w.scan_part = reinterpret_cast<uint32_t*>(b + P.off_scan_part);
+    w.gpart = reinterpret_cast<uint32_t*>(b + P.off_gpart);
+    w.tile_part = reinterpret_cast<uint32_t*>(b + P.off_tile_part);
     w.loss_part = reinterpret_cast<float*>(b + P.off_loss_part);
     return w;
 }
@@ -140,7 +141,7 @@ static bool plan_build(Plan& P, const int64_t* scene_n, int32_t n_scenes, const 
     cap = align_up((size_t)cap, kCapGranule);
     if (cap >= ((int64_t)1 << 31)) return false;
     P.cap = cap;
-    P.count_scan_parts = (pairs + kScanBlock - 1) / kScanBlock;
+    P.pair_groups = (pairs + kPairGroup - 1) / kPairGroup;
     P.tile_scan_parts = (tiles + kScanBlock - 1) / kScanBlock;
     P.raster_blocks = tiles;
     const int64_t loss_blocks = std::max<int64_t>((3 * pixels + 2047) / 2048, 2 * ssim_blocks(V));
@@ -169,7 +170,8 @@ static bool plan_build(Plan& P, const int64_t* scene_n, int32_t n_scenes, const 
     P.off_nlast = take(4 * (size_t)pixels);
     P.off_tfinal = take(4 * (size_t)pixels);
     P.off_gradrec = take(sizeof(GradRec) * (size_t)cap);
-    P.off_scan_part = take(4 * (size_t)(std::max(P.count_scan_parts, P.tile_scan_parts) + 1));
+    P.off_gpart = take(4 * (size_t)P.pair_groups);
+    P.off_tile_part = take(4 * 33 * (size_t)P.tile_scan_parts);
     P.off_loss_part = take(4 * (size_t)loss_blocks);
     P.ws_bytes = o;
     return true;

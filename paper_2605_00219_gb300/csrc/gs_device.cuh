@@ -366,70 +366,117 @@ __device__ __forceinline__ int tile_hi(float v, int T, int n)
 
 // Scan-line traversal (Sec. 4.1) of the tiles whose pixel-centre rectangle
 // meets the ellipse d^2 <= g.r2, band by band along the shorter dimension of
-// the tile bounding box: calls band(rows, coord, lo, hi) for every band that
-// meets a tile, in traversal order -- rows: bands are tile rows (coord = ty,
-// tiles tx = lo..hi), else tile columns (coord = tx, tiles ty = lo..hi).
+// the tile bounding box: rows -- bands are tile rows (coord = ty, tiles
+// tx = lo..hi), else tile columns (coord = tx, tiles ty = lo..hi).
+struct ScanLine {
+    bool rows;
+    int first, last;           // bands of the bounding box (empty: first > last)
+    float ex, ey, star, r2o;   // half-extents; offset of the band extreme; r2 x the other diagonal
+};
+
+__device__ __forceinline__ ScanLine scanline_setup(const BinGeom& g, int tw, int th, int TX, int TY)
+{
+    ScanLine L;
+    const float r2 = g.r2;
+    L.ex = FQ(FM(r2, g.a));
+    L.ey = FQ(FM(r2, g.c));
+    const int txl = tile_lo(FS(g.mx, L.ex), tw, TX), txh = tile_hi(FA(g.mx, L.ex), tw, TX);
+    const int tyl = tile_lo(FS(g.my, L.ey), th, TY), tyh = tile_hi(FA(g.my, L.ey), th, TY);
+    L.rows = tyh - tyl <= txh - txl;
+    L.first = L.rows ? tyl : txl;
+    L.last = L.rows ? tyh : txh;
+    if (txl > txh || tyl > tyh) L.last = L.first - 1;
+    L.star = FM(g.b, FQ(FD(r2, L.rows ? g.a : g.c)));
+    L.r2o = FM(r2, L.rows ? g.c : g.a);
+    return L;
+}
+
+// Tiles lo..hi of one band; false when it meets none.
+__device__ __forceinline__ bool scanline_band(const BinGeom& g, const ScanLine& L, int coord, int tw, int th, int TX,
+                                              int TY, int& lo, int& hi)
+{
+    const int tb = L.rows ? th : tw;                     // band width, and the mean along and across the bands
+    const float mb = L.rows ? g.my : g.mx, mo = L.rows ? g.mx : g.my;
+    const float eb = L.rows ? L.ey : L.ex, q = L.rows ? g.c : g.a;
+    const float d0 = FS(FA((float)(coord * tb), 0.5f), mb);
+    const float d1 = FS(FS((float)((coord + 1) * tb), 0.5f), mb);
+    const float dlo = fmaxf(d0, -eb), dhi = fminf(d1, eb);
+    if (!(dlo <= dhi)) return false;
+    const float dR = fminf(fmaxf(L.star, dlo), dhi);
+    const float dL = fminf(fmaxf(-L.star, dlo), dhi);
+    const float hR = FQ(fmaxf(0.0f, FM(g.det, FS(L.r2o, FM(dR, dR)))));
+    const float hL = FQ(fmaxf(0.0f, FM(g.det, FS(L.r2o, FM(dL, dL)))));
+    const float oR = FA(mo, FD(FA(FM(g.b, dR), hR), q));
+    const float oL = FA(mo, FD(FS(FM(g.b, dL), hL), q));
+    lo = tile_lo(oL, L.rows ? tw : th, L.rows ? TX : TY);
+    hi = tile_hi(oR, L.rows ? tw : th, L.rows ? TX : TY);
+    return lo <= hi;
+}
+
+// Every band that meets a tile, in traversal order: band(rows, coord, lo, hi).
 // Returns the number of tiles.
 template <typename Band>
-__device__ __forceinline__ uint32_t scanline_bands(const BinGeom& g, int tw, int th, int TX, int TY, Band band)
+__device__ __forceinline__ uint32_t scanline_bands(const BinGeom& g, const ScanLine& L, int tw, int th, int TX, int TY,
+                                                   Band band)
 {
-    const float r2 = g.r2;
-    float ex = FQ(FM(r2, g.a));
-    float ey = FQ(FM(r2, g.c));
-    int txl = tile_lo(FS(g.mx, ex), tw, TX), txh = tile_hi(FA(g.mx, ex), tw, TX);
-    int tyl = tile_lo(FS(g.my, ey), th, TY), tyh = tile_hi(FA(g.my, ey), th, TY);
-    if (txl > txh || tyl > tyh) return 0;
     uint32_t count = 0;
-    if (tyh - tyl <= txh - txl) {
-        float ystar = FM(g.b, FQ(FD(r2, g.a)));
-        float r2c = FM(r2, g.c);
-        for (int ty = tyl; ty <= tyh; ty++) {
-            float y0 = FS(FA((float)(ty * th), 0.5f), g.my);
-            float y1 = FS(FS((float)((ty + 1) * th), 0.5f), g.my);
-            float dlo = fmaxf(y0, -ey), dhi = fminf(y1, ey);
-            if (!(dlo <= dhi)) continue;
-            float dR = fminf(fmaxf(ystar, dlo), dhi);
-            float dL = fminf(fmaxf(-ystar, dlo), dhi);
-            float hR = FQ(fmaxf(0.0f, FM(g.det, FS(r2c, FM(dR, dR)))));
-            float hL = FQ(fmaxf(0.0f, FM(g.det, FS(r2c, FM(dL, dL)))));
-            float xR = FA(g.mx, FD(FA(FM(g.b, dR), hR), g.c));
-            float xL = FA(g.mx, FD(FS(FM(g.b, dL), hL), g.c));
-            int lo = tile_lo(xL, tw, TX), hi = tile_hi(xR, tw, TX);
-            if (lo > hi) continue;
-            band(true, ty, lo, hi);
-            count += (uint32_t)(hi - lo + 1);
-        }
-    } else {
-        float xstar = FM(g.b, FQ(FD(r2, g.c)));
-        float r2a = FM(r2, g.a);
-        for (int tx = txl; tx <= txh; tx++) {
-            float x0 = FS(FA((float)(tx * tw), 0.5f), g.mx);
-            float x1 = FS(FS((float)((tx + 1) * tw), 0.5f), g.mx);
-            float dlo = fmaxf(x0, -ex), dhi = fminf(x1, ex);
-            if (!(dlo <= dhi)) continue;
-            float dT = fminf(fmaxf(xstar, dlo), dhi);
-            float dB = fminf(fmaxf(-xstar, dlo), dhi);
-            float hT = FQ(fmaxf(0.0f, FM(g.det, FS(r2a, FM(dT, dT)))));
-            float hB = FQ(fmaxf(0.0f, FM(g.det, FS(r2a, FM(dB, dB)))));
-            float yT = FA(g.my, FD(FA(FM(g.b, dT), hT), g.a));
-            float yB = FA(g.my, FD(FS(FM(g.b, dB), hB), g.a));
-            int lo = tile_lo(yB, th, TY), hi = tile_hi(yT, th, TY);
-            if (lo > hi) continue;
-            band(false, tx, lo, hi);
-            count += (uint32_t)(hi - lo + 1);
-        }
+    for (int c = L.first; c <= L.last; c++) {
+        int lo, hi;
+        if (!scanline_band(g, L, c, tw, th, TX, TY, lo, hi)) continue;
+        band(L.rows, c, lo, hi);
+        count += (uint32_t)(hi - lo + 1);
     }
     return count;
 }
 
-// The same traversal tile by tile: emit(i, tile id) for the i-th tile.
-template <typename Emit>
-__device__ __forceinline__ uint32_t scanline_tiles(const BinGeom& g, int tw, int th, int TX, int TY, Emit emit)
+// The traversal of one pair by a whole warp (every lane with the same g): the
+// lanes take a band each, then the tiles of those bands in order, 32 at a time:
+// emit(i, tile id) for the i-th tile.  first2(k, coord, lo, hi) is called by every
+// lane for the first two bands that meet a tile.  Returns the tiles, and in nb the bands.
+// A lane that walked a footprint of a thousand tiles alone held its block for the
+// whole kernel's time.
+template <typename First2, typename Emit>
+__device__ __forceinline__ uint32_t warp_scanline(const BinGeom& g, int tw, int th, int TX, int TY, uint32_t& nb,
+                                                  First2 first2, Emit emit)
 {
-    uint32_t i = 0;
-    return scanline_bands(g, tw, th, TX, TY, [&](bool rows, int coord, int lo, int hi) {
-        for (int t = lo; t <= hi; t++, i++) emit(i, rows ? (uint32_t)(coord * TX + t) : (uint32_t)(t * TX + coord));
-    });
+    const ScanLine L = scanline_setup(g, tw, th, TX, TY);
+    const int lane = threadIdx.x & 31;
+    uint32_t count = 0;
+    nb = 0;
+    for (int c0 = L.first; c0 <= L.last; c0 += 32) {
+        int lo = 0, hi = -1;
+        const int c = c0 + lane;
+        if (c > L.last || !scanline_band(g, L, c, tw, th, TX, TY, lo, hi)) lo = 0, hi = -1;
+        const uint32_t n = (uint32_t)(hi - lo + 1);
+        uint32_t x = n;         // inclusive sum over the bands
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        for (uint32_t m = __ballot_sync(0xffffffffu, n != 0u); m && nb < 3u; m &= m - 1u, nb++) {
+            const int k = __ffs(m) - 1;
+            const int l = __shfl_sync(0xffffffffu, lo, k), h = __shfl_sync(0xffffffffu, hi, k);
+            if (nb < 2u) first2(nb, L.rows, c0 + k, l, h);
+        }
+        const uint32_t total = __shfl_sync(0xffffffffu, x, 31);
+        for (uint32_t i0 = 0; i0 < total; i0 += 32) {
+            const uint32_t i = i0 + lane;
+            int k = 0;          // the band of tile i: the first with x > i
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(0xffffffffu, x, k + o - 1) <= i) k += o;
+            const uint32_t xk = __shfl_sync(0xffffffffu, x, k & 31);
+            const int hk = __shfl_sync(0xffffffffu, hi, k & 31);
+            if (i < total) {
+                const uint32_t t = (uint32_t)hk - (xk - 1u - i);
+                const uint32_t cd = (uint32_t)(c0 + k);
+                emit(count + i, L.rows ? cd * TX + t : t * TX + cd);
+            }
+        }
+        count += total;
+    }
+    return count;
 }
 
 // Tile span of a pair, written by the projection's traversal and read by

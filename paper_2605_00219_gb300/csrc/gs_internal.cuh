@@ -24,6 +24,9 @@ constexpr int kScanThreads = 512;
 constexpr int kScanItems = 8;
 constexpr int kScanBlock = kScanThreads * kScanItems;
 
+// Pairs per partial sum of the emission-slot scan (one warp sums them).
+constexpr int kPairGroup = 1024;
+
 // Raster backward block: 4 warps.
 constexpr int kBwdThreads = 128;
 
@@ -35,7 +38,7 @@ struct Plan {
     int64_t cap;                 // intersection capacity
     gs_tuning tuning;
     int32_t sh_bf16, mom_bf16;
-    int64_t count_scan_parts;    // ceil(pairs / kScanBlock)
+    int64_t pair_groups;         // ceil(pairs / kPairGroup)
     int64_t tile_scan_parts;     // ceil(tiles / kScanBlock)
     int64_t raster_blocks;       // total tiles
     int32_t sm_count;            // SMs of the device current at plan creation (152 if none)
@@ -43,7 +46,7 @@ struct Plan {
     size_t off_hdr, off_count, off_offset, off_rec, off_span, off_rank;
     size_t off_bucket, off_keys, off_vals, off_pid, off_pid_sorted;
     size_t off_tile_cnt, off_tile_cur;
-    size_t off_ranges, off_nlast, off_tfinal, off_gradrec, off_scan_part, off_loss_part, off_order;
+    size_t off_ranges, off_nlast, off_tfinal, off_gradrec, off_gpart, off_tile_part, off_loss_part, off_order;
     size_t ws_bytes;
 };
 
@@ -67,7 +70,8 @@ struct WsPtrs {
     uint32_t* nlast;
     float* tfinal;
     GradRec* gradrec;
-    uint32_t* scan_part;
+    uint32_t* gpart;           // intersections per kPairGroup pairs, then their exclusive scan
+    uint32_t* tile_part;       // per 4,096 tiles: intersections, then tiles per list-length bucket (32)
     float* loss_part;
 };
 

@@ -39,7 +39,8 @@ __device__ __forceinline__ void project_pair(const ViewDesc& vd, int tw, int th,
     const uint32_t TX = (uint32_t)vd.TX;
     uint32_t* __restrict__ to = tile_over + vd.tile_base;
     if (bg.valid)
-        cnt = scanline_bands(bg, tw, th, vd.TX, vd.TY, [&](bool rw, int coord, int lo, int hi) {
+        cnt = scanline_bands(bg, scanline_setup(bg, tw, th, vd.TX, vd.TY), tw, th, vd.TX, vd.TY,
+                             [&](bool rw, int coord, int lo, int hi) {
             rows = rw;
             const uint32_t pk = (uint32_t)lo | ((uint32_t)hi << 16);
             if (nb == 0) { c0 = (uint32_t)coord; r0 = pk; }
