@@ -266,6 +266,14 @@ gs_status gs_project_bwd_adam(const gs_plan* plan, void* ws, const gs_scene_buf*
                               const float* cams, const gs_adam* adam, float* grads_out,
                               void* stream);
 
+/* The gradient-only mode of gs_project_bwd_adam with the results where a
+ * framework wants them: for every scene, the gradient with respect to the stored
+ * parameters in the layout of its buffers -- grads[s].geom: float4[3][n],
+ * grads[s].sh: float4[12][n], or uint4[6][n] (BF16 storage, rounded to nearest) --
+ * with grads[s].n = the scene's n; the other fields are ignored. */
+gs_status gs_project_bwd_grads(const gs_plan* plan, void* ws, const gs_scene_buf* scenes,
+                               const float* cams, const gs_scene_buf* grads, void* stream);
+
 /* Advance the workspace Adam step counter by one (for graph replay). */
 gs_status gs_adam_advance(const gs_plan* plan, void* ws, void* stream);
 

@@ -3,7 +3,7 @@
 `Renderer.render(scenes)` returns the rendered views as a differentiable
 tensor (pixels x 3, views concatenated).  Its backward runs the library's
 own rasterization backward and projection backward (gs_raster_bwd, then
-gs_project_bwd_adam in gradient-only mode); nothing is differentiated by
+gs_project_bwd_grads); nothing is differentiated by
 torch.  Transmittance is recomputed in the backward from the per-pixel final
 transmittance, not stored per pair.
 
@@ -88,17 +88,8 @@ class _GSRender(torch.autograd.Function):
         (image,) = ctx.saved_tensors
         dl = grad_image.contiguous().float()
         gsstep.gs_raster_bwd(r.plan, r.ws, image, dl)
-        N = sum(r.scene_sizes)
-        go = torch.empty((15, N, 4), dtype=torch.float32, device=r.device)
-        gsstep.gs_project_bwd_adam(r.plan, r.ws, ctx.bufs, r.cams, None, go)
-        grads = [None]
-        base = 0
-        for b in ctx.bufs:
-            n = b.n
-            dgeom = go[0:3, base:base + n].contiguous()
-            dsh = go[3:15, base:base + n]
-            if b.sh.dtype == torch.bfloat16:
-                dsh = dsh.reshape(6, 2, n, 4).permute(0, 2, 1, 3).reshape(6, n, 8).to(torch.bfloat16)
-            grads += [dgeom, dsh.contiguous()]
-            base += n
-        return tuple(grads)
+        # the library writes each scene's gradients in the layout and type of its
+        # stored tensors
+        grads = [(torch.empty_like(b.geom), torch.empty_like(b.sh)) for b in ctx.bufs]
+        gsstep.gs_project_bwd_grads(r.plan, r.ws, ctx.bufs, r.cams, grads)
+        return (None, *(t for pair in grads for t in pair))

@@ -412,6 +412,26 @@ gs_status gs_project_bwd_adam(const gs_plan* plan, void* ws, const gs_scene_buf*
     return launch_status();
 }
 
+gs_status gs_project_bwd_grads(const gs_plan* plan, void* ws, const gs_scene_buf* scenes, const float* cams,
+                               const gs_scene_buf* grads, void* stream)
+{
+    const StageRange range("gs_project_bwd_grads");
+    if (!plan || !ws || !cams) return GS_ERR_INVALID_ARG;
+    const Plan& P = plan->p;
+    gs_status e = check_scenes(P, scenes, false);
+    if (e == GS_OK) e = check_scenes(P, grads, false);
+    if (e != GS_OK) return e;
+    WsPtrs w = carve(P, ws);
+    Scenes S = make_scenes(P, scenes);
+    for (int s = 0; s < P.n_scenes; s++) {
+        S.s[s].stats = nullptr;
+        S.s[s].dgeom = static_cast<float4*>(grads[s].geom);
+        S.s[s].dsh = grads[s].sh;
+    }
+    launch_project_bwd_adam(P, S, cams, w, nullptr, nullptr, static_cast<cudaStream_t>(stream));
+    return launch_status();
+}
+
 gs_status gs_adam_advance(const gs_plan* plan, void* ws, void* stream)
 {
     if (!plan || !ws) return GS_ERR_INVALID_ARG;

@@ -50,6 +50,8 @@ struct SceneDesc {
     void* m;               // float4[15][n] or uint2[15][n]
     void* v;
     float2* stats;         // NULL or densification statistics, float2[n]
+    float4* dgeom;         // NULL, or the scene's gradients in the layout of geom and sh
+    void* dsh;
 };
 
 struct Scenes {

@@ -292,6 +292,14 @@ __device__ __forceinline__ uint32_t bf16x2_sr(float lo, float hi, uint32_t rbits
     return d;
 }
 
+// bf16 pair by rounding to nearest even
+__device__ __forceinline__ uint32_t bf16x2_rn(float lo, float hi)
+{
+    uint32_t d;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+    return d;
+}
+
 // Per-thread stream key: one hash of (seed, step, Gaussian), uniform over
 // 32 bits.  Draw ctr of the stream is one multiply-xorshift round of
 // key + ctr * 0x9E3779B9: for each ctr a bijection of the key, hence uniform
@@ -480,7 +488,11 @@ __global__ void __launch_bounds__(kPbaThreads, 4) k_project_bwd_adam(Views V, Sc
             st.y += st_cnt;
             sc.stats[g] = st;
         }
-        if (A.grad_only) {
+        if (A.grad_only && sc.dgeom) {
+            sc.dgeom[g] = make_float4(dmu[0], dmu[1], dmu[2], 0.f);
+            sc.dgeom[n + g] = make_float4(dq[0], dq[1], dq[2], dq[3]);
+            sc.dgeom[2 * n + g] = make_float4(ds[0], ds[1], ds[2], dop);
+        } else if (A.grad_only) {
             const int64_t N = S.total;
             grads_out[0 * N + gi] = make_float4(dmu[0], dmu[1], dmu[2], 0.f);
             grads_out[1 * N + gi] = make_float4(dq[0], dq[1], dq[2], dq[3]);
@@ -527,6 +539,22 @@ __global__ void __launch_bounds__(kPbaThreads, 4) k_project_bwd_adam(Views V, Sc
     const SceneDesc& sc = S.s[s];
     const int64_t g = gi - sc.base;
     const int64_t n = sc.n;
+    if (A.grad_only && sc.dgeom) {
+        // in the stored layout (a separate pass over float4[15][N] to split, permute
+        // and convert it cost twice the gradients' bytes)
+        if (SH16) {
+#pragma unroll
+            for (int jp = 0; jp < 6; jp++) {
+                const float4 a = sG[tid][2 * jp], b = sG[tid][2 * jp + 1];
+                reinterpret_cast<uint4*>(sc.dsh)[(int64_t)jp * n + g] =
+                    make_uint4(bf16x2_rn(a.x, a.y), bf16x2_rn(a.z, a.w), bf16x2_rn(b.x, b.y), bf16x2_rn(b.z, b.w));
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 12; j++) reinterpret_cast<float4*>(sc.dsh)[(int64_t)j * n + g] = sG[tid][j];
+        }
+        return;
+    }
     if (A.grad_only) {
         const int64_t N = S.total;
 #pragma unroll
@@ -604,7 +632,7 @@ void launch_project_bwd_adam(const Plan& P, const Scenes& S, const float* cams, 
     A.b2 = adam ? adam->beta2 : 0.999f;
     A.eps = adam ? adam->eps : 1e-15f;
     A.step = adam ? adam->step : 1;
-    A.grad_only = grads_out != nullptr;
+    A.grad_only = adam == nullptr || grads_out != nullptr;
     A.seed = adam ? adam->seed : 0u;
     const int64_t blocks = (S.total + kPbaThreads - 1) / kPbaThreads;
 #define GS_PBA(SH, MO)                                                                                              \

@@ -34,7 +34,8 @@ STATUS_NAMES = {0: "GS_OK", 1: "GS_ERR_INVALID_ARG", 2: "GS_ERR_CAPACITY", 3: "G
 # exported symbols (the C ABI)
 SYMBOLS = ["gs_plan_create", "gs_plan_destroy", "gs_workspace_bytes", "gs_plan_query", "gs_workspace_init",
            "gs_project_fwd", "gs_bin_sort", "gs_raster_fwd", "gs_loss_l1", "gs_raster_bwd",
-           "gs_project_bwd_adam", "gs_adam_advance", "gs_read_stats", "gs_workspace_buffer", "gs_status_str",
+           "gs_project_bwd_adam", "gs_project_bwd_grads", "gs_adam_advance", "gs_read_stats", "gs_workspace_buffer",
+           "gs_status_str",
            "gs_loss_l1_noalloc", "gs_loss_l1_ssim", "gs_loss_l1_ssim_masked", "gs_densify_scratch_bytes", "gs_densify_count",
            "gs_densify_counts", "gs_densify_apply", "gs_reset_opacity", "gs_workspace_set_step"]
 L1_NOALLOC_MAX_VALUES = 67108864
@@ -105,6 +106,7 @@ def lib():
         L.gs_loss_l1_ssim_masked.argtypes = [vp, vp, vp, vp, ctypes.c_float, vp, vp]
         L.gs_raster_bwd.argtypes = [vp, vp, vp, vp, vp]
         L.gs_project_bwd_adam.argtypes = [vp, vp, ctypes.POINTER(gs_scene_buf), vp, ctypes.POINTER(gs_adam), vp, vp]
+        L.gs_project_bwd_grads.argtypes = [vp, vp, ctypes.POINTER(gs_scene_buf), vp, ctypes.POINTER(gs_scene_buf), vp]
         L.gs_adam_advance.argtypes = [vp, vp, vp]
         L.gs_workspace_set_step.argtypes = [vp, vp, i32, vp]
         L.gs_read_stats.argtypes = [vp, vp, ctypes.POINTER(gs_stats), vp]
@@ -123,7 +125,7 @@ def lib():
         L.gs_status_str.restype = ctypes.c_char_p
         for name in ["gs_workspace_init", "gs_project_fwd", "gs_bin_sort", "gs_raster_fwd", "gs_loss_l1",
                      "gs_loss_l1_ssim", "gs_loss_l1_ssim_masked", "gs_raster_bwd", "gs_project_bwd_adam",
-                     "gs_adam_advance", "gs_read_stats",
+                     "gs_project_bwd_grads", "gs_adam_advance", "gs_read_stats",
                      "gs_densify_count", "gs_densify_counts", "gs_densify_apply", "gs_reset_opacity",
                      "gs_workspace_set_step"]:
             getattr(L, name).restype = ctypes.c_int
@@ -137,14 +139,20 @@ def _check(rc: int, what: str):
 
 
 def _ptr(t):
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+# the current stream's handle without building a Stream object (a third of a
+# small eager call's host time went there)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(torch._C._cuda_getDevice())
+    return torch.cuda.current_stream().cuda_stream
 
 
 class Plan:
@@ -259,6 +267,16 @@ def gs_project_bwd_adam(plan: Plan, ws, scenes, cams, adam: gs_adam | None, grad
     _check(lib().gs_project_bwd_adam(plan.handle, _ptr(ws), scene_bufs(scenes), _ptr(cams),
                                      ctypes.byref(adam) if adam is not None else None, _ptr(grads_out),
                                      _stream(stream)), "gs_project_bwd_adam")
+
+
+def gs_project_bwd_grads(plan: Plan, ws, scenes, cams, grads, stream=None):
+    """grads: one (geom, sh) tensor pair per scene, written in the layout of the
+    scene's buffers (SH in its storage type)."""
+    arr = (gs_scene_buf * len(grads))()
+    for i, (b, (dgeom, dsh)) in enumerate(zip(scenes, grads)):
+        arr[i] = gs_scene_buf(b.n, dgeom.data_ptr(), dsh.data_ptr(), None, None, None)
+    _check(lib().gs_project_bwd_grads(plan.handle, _ptr(ws), scene_bufs(scenes), _ptr(cams), arr, _stream(stream)),
+           "gs_project_bwd_grads")
 
 
 def gs_adam_advance(plan: Plan, ws, stream=None):
