@@ -17,14 +17,14 @@
 //   generate keys: from the tile spans the projection kept, each intersection
 //                  goes to its rank's or the next free place of its tile (depth
 //                  code and emission slot), and its pair to the emission slot
-//   sorting      : one thread block per tile sorts the tile's entries by
-//                  (depth code, emission slot) -- unique, so the arrival
-//                  order of the atomics does not matter -- and writes the
-//                  keys, emission slots and pairs: a block merge sort in
-//                  shared memory up to kTileSortMax entries; longer lists
-//                  are sorted in chunks of that size and merged in global
-//                  memory by rank (each entry's position in the other run by
-//                  binary search)
+//   sorting      : a thread block, a part of one or a warp sorts a tile's
+//                  entries by (depth code, emission slot) -- unique, so the
+//                  arrival order of the atomics does not matter -- and writes
+//                  the keys, emission slots and pairs: 32-bit words of depth
+//                  code and arrival index sorted in registers and merged in
+//                  shared memory, ties put in order afterwards; 64-bit keys
+//                  where the words are too short; longer lists in chunks,
+//                  merged in global memory piece by piece
 // K never leaves the device: every kernel reads it from the workspace header
 // and grids are sized by the plan.  When K exceeds the capacity nothing is
 // emitted and every tile list is empty (GS_STATUS_CAPACITY reports it).
@@ -493,9 +493,10 @@ __device__ __forceinline__ unsigned long long sort_key(uint32_t low, uint32_t e)
 // that warp reads and writes them, so the level synchronises the warp; a
 // level that reads wider runs synchronises the group, also before its
 // reads.  The caller synchronises the group before.
-__device__ __forceinline__ void cmpx(unsigned long long& a, unsigned long long& b)
+template <typename Key>
+__device__ __forceinline__ void cmpx(Key& a, Key& b)
 {
-    const unsigned long long lo = a < b ? a : b, hi = a < b ? b : a;
+    const Key lo = a < b ? a : b, hi = a < b ? b : a;
     a = lo;
     b = hi;
 }
@@ -512,34 +513,37 @@ struct SortGroup {
     }
 };
 
+// Whether any thread of the group has the flag (synchronises the group).
+__device__ __forceinline__ bool group_any(const SortGroup& g, bool flag)
+{
+    if (g.n == 32) return __any_sync(0xffffffffu, flag);
+    if (g.bar == 0) return __syncthreads_or(flag);
+    uint32_t r;
+    asm volatile(
+        "{\n.reg .pred p, q;\nsetp.ne.u32 q, %1, 0;\nbar.red.or.pred p, %2, %3, q;\nselp.u32 %0, 1, 0, p;\n}"
+        : "=r"(r)
+        : "r"((uint32_t)flag), "r"(g.bar), "r"(g.n)
+        : "memory");
+    return r != 0;
+}
+
 __device__ __forceinline__ SortGroup whole_block() { return SortGroup{(int)threadIdx.x, (int)blockDim.x, 0}; }
 
-__device__ void block_merge_sort_smem(unsigned long long* s, int N, const SortGroup& g)
+// Merge levels of the block merge sort from run width w0 (every run of w0 keys
+// sorted, the group synchronised): threads t < N / IT place IT outputs each.
+template <int IT, typename Key>
+__device__ __forceinline__ void merge_levels_smem(Key* s, int N, int w0, const SortGroup& g)
 {
-    constexpr int IT = 8;
     const int nt = N / IT, t = g.t;
-    unsigned long long r[IT];
-    if (t < nt) {
-#pragma unroll
-        for (int k = 0; k < IT; k++) r[k] = s[IT * t + k];
-        cmpx(r[0], r[1]); cmpx(r[2], r[3]); cmpx(r[4], r[5]); cmpx(r[6], r[7]);
-        cmpx(r[0], r[2]); cmpx(r[1], r[3]); cmpx(r[4], r[6]); cmpx(r[5], r[7]);
-        cmpx(r[1], r[2]); cmpx(r[5], r[6]);
-        cmpx(r[0], r[4]); cmpx(r[1], r[5]); cmpx(r[2], r[6]); cmpx(r[3], r[7]);
-        cmpx(r[2], r[4]); cmpx(r[3], r[5]);
-        cmpx(r[1], r[2]); cmpx(r[3], r[4]); cmpx(r[5], r[6]);
-#pragma unroll
-        for (int k = 0; k < IT; k++) s[IT * t + k] = r[k];
-    }
-    __syncwarp();
-    for (int w = IT; w < N; w <<= 1) {
+    Key r[IT];
+    for (int w = w0; w < N; w <<= 1) {
         const bool in_warp = 2 * w <= 32 * IT;
         const int base = (IT * t) & ~(2 * w - 1), diag = IT * t - base;
         const int la = min(w, N - base), lb = max(0, min(w, N - base - w));
         const bool merge = t < nt && lb > 0;   // a lone last run stays in place
         if (merge) {
-            const unsigned long long* A = s + base;
-            const unsigned long long* B = s + base + w;
+            const Key* A = s + base;
+            const Key* B = s + base + w;
             int lo = max(0, diag - lb), hi = min(diag, la);
             while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
@@ -547,25 +551,31 @@ __device__ void block_merge_sort_smem(unsigned long long* s, int N, const SortGr
                 else hi = mid;
             }
             int a = lo, b = diag - lo;
-            unsigned long long ha = a < la ? A[a] : 0ull, hb = b < lb ? B[b] : 0ull;
+            Key ha = a < la ? A[a] : Key(0), hb = b < lb ? B[b] : Key(0);
 #pragma unroll
             for (int k = 0; k < IT; k++) {
                 const bool take_a = b >= lb || (a < la && ha <= hb);
                 r[k] = take_a ? ha : hb;
                 if (take_a) {
                     a++;
-                    ha = a < la ? A[a] : 0ull;
+                    ha = a < la ? A[a] : Key(0);
                 } else {
                     b++;
-                    hb = b < lb ? B[b] : 0ull;
+                    hb = b < lb ? B[b] : Key(0);
                 }
             }
         }
         if (in_warp) __syncwarp();
         else g.sync();
         if (merge) {
+            if constexpr (sizeof(Key) == 4) {
 #pragma unroll
-            for (int k = 0; k < IT; k++) s[IT * t + k] = r[k];
+                for (int k = 0; k < IT; k += 4)
+                    *reinterpret_cast<uint4*>(s + IT * t + k) = make_uint4(r[k], r[k + 1], r[k + 2], r[k + 3]);
+            } else {
+#pragma unroll
+                for (int k = 0; k < IT; k++) s[IT * t + k] = r[k];
+            }
         }
         // the next level (width 2w) reads other warps' keys unless its runs
         // still fit in one warp
@@ -573,6 +583,61 @@ __device__ void block_merge_sort_smem(unsigned long long* s, int N, const SortGr
         else g.sync();
     }
     g.sync();
+}
+
+template <typename Key>
+__device__ __forceinline__ void sort8(Key* r)
+{
+    cmpx(r[0], r[1]); cmpx(r[2], r[3]); cmpx(r[4], r[5]); cmpx(r[6], r[7]);
+    cmpx(r[0], r[2]); cmpx(r[1], r[3]); cmpx(r[4], r[6]); cmpx(r[5], r[7]);
+    cmpx(r[1], r[2]); cmpx(r[5], r[6]);
+    cmpx(r[0], r[4]); cmpx(r[1], r[5]); cmpx(r[2], r[6]); cmpx(r[3], r[7]);
+    cmpx(r[2], r[4]); cmpx(r[3], r[5]);
+    cmpx(r[1], r[2]); cmpx(r[3], r[4]); cmpx(r[5], r[6]);
+}
+
+__device__ void block_merge_sort_smem(unsigned long long* s, int N, const SortGroup& g)
+{
+    constexpr int IT = 8;
+    unsigned long long r[IT];
+    if (g.t < N / IT) {
+#pragma unroll
+        for (int k = 0; k < IT; k++) r[k] = s[IT * g.t + k];
+        sort8(r);
+#pragma unroll
+        for (int k = 0; k < IT; k++) s[IT * g.t + k] = r[k];
+    }
+    __syncwarp();
+    merge_levels_smem<IT>(s, N, IT, g);
+}
+
+// Ascending sort of a warp's 256 keys in registers, lane l holding [8l, 8l + 8):
+// 8 keys by the network, then bitonic merges of run width 8, 16, ... up to `most`
+// keys, which lie in the first most / 8 lanes (each: the mirrored exchange, then halving exchanges, across lanes by shuffles
+// and within a lane in registers).  No shared-memory round trips.
+__device__ __forceinline__ void warp_sort256(uint32_t* r, int lane, int most)
+{
+    sort8(r);
+#pragma unroll
+    for (int w = 1; w < 32; w <<= 1) {          // run width in lanes
+        if (8 * w >= most) break;
+        uint32_t y[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) y[k] = __shfl_xor_sync(0xffffffffu, r[7 - k], 2 * w - 1);
+#pragma unroll
+        for (int k = 0; k < 8; k++) r[k] = (lane & w) ? max(r[k], y[k]) : min(r[k], y[k]);
+#pragma unroll
+        for (int d = w >> 1; d > 0; d >>= 1)
+#pragma unroll
+            for (int k = 0; k < 8; k++) {
+                const uint32_t z = __shfl_xor_sync(0xffffffffu, r[k], d);
+                r[k] = (lane & d) ? max(r[k], z) : min(r[k], z);
+            }
+#pragma unroll
+        for (int k = 0; k < 4; k++) cmpx(r[k], r[k + 4]);
+        cmpx(r[0], r[2]); cmpx(r[1], r[3]); cmpx(r[4], r[6]); cmpx(r[5], r[7]);
+        cmpx(r[0], r[1]); cmpx(r[2], r[3]); cmpx(r[4], r[5]); cmpx(r[6], r[7]);
+    }
 }
 
 // (depth code, emission slot) lists in two layouts: one uint2 per entry, or
@@ -589,48 +654,155 @@ struct SplitList {
     __device__ void put(uint32_t i, unsigned long long x) const { k[i] = (uint32_t)(x >> 32); v[i] = (uint32_t)x; }
 };
 
-// Entries of a sorted run [b, b + len) below key x (binary search; keys
-// unique).
-template <class L>
-__device__ __forceinline__ uint32_t rank_in_run(const L& l, uint32_t b, uint32_t len, unsigned long long x)
-{
-    uint32_t lo = 0, hi = len;
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (l.get(b + mid) < x) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-
-// One merge level of run width `run` over a list of n entries at s0: each
-// entry goes to its index in its own run plus its rank in the other run.
+// One merge level of run width `run` (a power of two, at least kTileSortMax) over a
+// list of n entries at s0, kTileSortMax outputs at a time: where each such piece
+// starts in its two runs by one binary search per thread, all at once; then both parts
+// of a piece read to shared memory and merged there, 8 outputs a thread.  (A search
+// per entry in global memory took 165 us a level for a list of 21,000.)
 template <class Src, class Dst>
-__device__ void merge_level(const Src& src, const Dst& dst, uint32_t s0, uint32_t n, uint32_t run)
+__device__ void merge_level(const Src& src, const Dst& dst, uint32_t s0, uint32_t n, uint32_t run,
+                            unsigned long long* sk, uint32_t* split)
 {
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-        const uint32_t ri = i / run, b = (ri & ~1u) * run;
-        const unsigned long long x = src.get(s0 + i);
-        uint32_t pos;
-        if ((ri & 1u) == 0) {   // left run: rank among the right run
-            const uint32_t pb = b + run, plen = pb < n ? min(run, n - pb) : 0u;
-            pos = i + (plen ? rank_in_run(src, s0 + pb, plen, x) : 0u);
-        } else {                // right run: rank among the left run
-            pos = b + (i - ri * run) + rank_in_run(src, s0 + b, run, x);
+    constexpr uint32_t P = kTileSortMax, IT = 8;
+    static_assert(P == IT * kTileSortThreads, "every thread merges 8 outputs of a piece");
+    const uint32_t pieces = (n + P - 1) / P;
+    for (uint32_t j0 = 0; j0 < pieces; j0 += kTileSortThreads) {
+        for (uint32_t j = j0 + threadIdx.x; j <= j0 + kTileSortThreads && j < pieces; j += blockDim.x) {
+            const uint32_t base = (j * P) & ~(2u * run - 1u), diag = j * P - base;
+            const uint32_t la = min(run, n - base), lb = min(run, n - base - la);
+            uint32_t lo = diag > lb ? diag - lb : 0u, hi = min(diag, la);
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (src.get(s0 + base + mid) < src.get(s0 + base + la + diag - 1u - mid)) lo = mid + 1u;
+                else hi = mid;
+            }
+            split[j - j0] = lo;
         }
-        dst.put(s0 + pos, x);
+        __syncthreads();
+        const uint32_t j1 = min(pieces, j0 + (uint32_t)kTileSortThreads);
+        for (uint32_t j = j0; j < j1; j++) {
+            const uint32_t base = (j * P) & ~(2u * run - 1u), diag = j * P - base;
+            const uint32_t la = min(run, n - base), lb = min(run, n - base - la);
+            const uint32_t end = min(diag + P, la + lb);
+            const uint32_t a0 = split[j - j0], a1 = end < la + lb ? split[j + 1 - j0] : la;
+            const uint32_t b0 = diag - a0, b1 = end - a1, na = a1 - a0, m = end - diag;
+#pragma unroll
+            for (uint32_t k = 0; k < IT; k++) {
+                const uint32_t i = threadIdx.x + k * kTileSortThreads;
+                if (i < m) sk[i] = src.get(s0 + base + (i < na ? a0 + i : la + b0 + i - na));
+            }
+            __syncthreads();
+            const uint32_t nb = b1 - b0, d = min(IT * threadIdx.x, m);
+            uint32_t lo = d > nb ? d - nb : 0u, hi = min(d, na);
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (sk[mid] < sk[na + d - 1u - mid]) lo = mid + 1u;
+                else hi = mid;
+            }
+            uint32_t a = lo, b = d - lo;
+#pragma unroll
+            for (uint32_t k = 0; k < IT; k++) {
+                if (d + k >= m) break;
+                const unsigned long long ha = a < na ? sk[a] : ~0ull, hb = b < nb ? sk[na + b] : ~0ull;
+                const bool take_a = b >= nb || (a < na && ha < hb);
+                dst.put(s0 + base + diag + d + k, take_a ? ha : hb);
+                a += take_a ? 1u : 0u;
+                b += take_a ? 0u : 1u;
+            }
+            __syncthreads();
+        }
     }
-    __syncthreads();
 }
 
-// One thread block per tile (launched longest lists first).  Input: the
-// tile's bucket [s0, s1) of (depth code, emission slot) in atomic arrival
+// The tile sort (longest lists launched first).  Input: the tile's bucket [s0, s1) of (depth code, emission slot) in atomic arrival
 // order.  Output at the same positions: keys_sorted = tile << shift | depth
 // code, vals_sorted = emission slot, pid_sorted = the slot's pair.
 //
-// One tile's list of n <= 8 g.n entries, sorted in shared memory (sk) by the
-// group g.
-__device__ __forceinline__ void tile_sort_group(const Views& V, int64_t gt, uint32_t s0, uint32_t n, unsigned long long* sk,
+// A run of n <= IT g.n entries at b, sorted by the group on 32-bit words (depth code,
+// arrival index) where the two fit: 256 words at a time sorted in a warp's registers,
+// wider runs by merges in shared memory (`key`: IT g.n words).  Equal depth codes (17%
+// of the entries at 3M Gaussians, 1080p, in runs of two or three) then still have
+// arrival order, and each entry of a run counts the run's smaller emission slots.
+// put(position, depth code, emission slot, pair(slot)) takes the sorted entries.  False, with
+// nothing put, if `bits` of depth code leave no room for the index or more than
+// kTieRun entries share a code: the caller sorts 64-bit keys then.
+constexpr int kTieRun = 32;
+
+template <int IT, typename Pair, typename Put>
+__device__ __forceinline__ bool sort_words(const uint2* b, int n, int bits, uint32_t* key, const SortGroup& g, Pair pair,
+                                           Put put)
+{
+    const int ib = 32 - __clz((n - 1) | 1);        // bits of the arrival index
+    if (bits + ib > 32) return false;
+    const int lane = g.t & 31;
+#pragma unroll
+    for (int c = 0; c < IT / 8; c++) {
+        const int w0 = (g.t >> 5) * 32 * IT + 256 * c;
+        if (w0 >= n) break;
+        // the entries dealt to the first L lanes only, so a short list needs only
+        // the merges of L lanes (the others hold padding)
+        const int m = min(n - w0, 256);
+        const int L = m <= 8 ? 1 : 1 << (32 - __clz((m - 1) >> 3));
+        uint32_t r[8];
+        uint2 q[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            const int i = L * k + lane;
+            q[k] = lane < L && i < m ? b[w0 + i] : make_uint2(0u, 0u);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            const int i = L * k + lane;
+            const bool in = lane < L && i < m;
+            r[k] = in ? (q[k].x << ib) | (uint32_t)(w0 + i) : ~0u;
+            if (IT == 8 && in) key[IT * g.n + w0 + i] = q[k].y;
+        }
+        warp_sort256(r, lane, 8 * L);
+        reinterpret_cast<uint4*>(key + w0 + 8 * lane)[0] = make_uint4(r[0], r[1], r[2], r[3]);
+        reinterpret_cast<uint4*>(key + w0 + 8 * lane)[1] = make_uint4(r[4], r[5], r[6], r[7]);
+    }
+    g.sync();
+    if (n > 256) merge_levels_smem<IT>(key, (n + IT - 1) / IT * IT, 256, g);
+    bool far = false;
+    for (int i = g.t; i + kTieRun < n; i += g.n) far |= key[i] >> ib == key[i + kTieRun] >> ib;
+    if (group_any(g, far)) return false;
+    const uint32_t im = (1u << ib) - 1u;
+    auto slot = [&](uint32_t i) { return IT == 8 ? key[IT * g.n + i] : b[i].y; };
+    constexpr int F = IT / 8;                      // entries in flight per thread (4 took 10% more)
+    for (int i0 = g.t; i0 < n; i0 += F * g.n) {
+        uint32_t x[F], e[F], p[F];
+#pragma unroll
+        for (int k = 0; k < F; k++) {
+            const int i = i0 + k * g.n;
+            x[k] = i < n ? key[i] : 0u;
+            e[k] = i < n ? slot(x[k] & im) : 0u;
+        }
+#pragma unroll
+        for (int k = 0; k < F; k++) p[k] = i0 + k * g.n < n ? pair(e[k]) : 0u;
+#pragma unroll
+        for (int k = 0; k < F; k++) {
+            const int i = i0 + k * g.n;
+            if (i >= n) break;
+            const uint32_t low = x[k] >> ib;
+            int first = i, pos = i;
+            while (first > 0 && key[first - 1] >> ib == low) first--;
+            if (first < i || (i + 1 < n && key[i + 1] >> ib == low)) {
+                pos = first;
+                for (int j = first; j < n && key[j] >> ib == low; j++) pos += slot(key[j] & im) < e[k];
+            }
+            put(pos, low, e[k], p[k]);
+        }
+    }
+    return true;
+}
+
+// One tile's list of n <= IT g.n entries, sorted by the group g in shared memory
+// (sk: 4 IT g.n bytes, 8 of them for each entry where 64-bit keys may be sorted,
+// n <= 8 g.n).  Words where they serve, 64-bit keys otherwise; false if neither.
+// 3M Gaussians, 4x1080p, all lists: 462 us with 64-bit keys, 257 us; without the
+// emission slots in shared memory (IT = 8) 10% more.
+template <int IT>
+__device__ __forceinline__ bool tile_sort_group(const Views& V, int64_t gt, uint32_t s0, uint32_t n, unsigned long long* sk,
                                 const SortGroup& g, uint2* bucket, const uint32_t* __restrict__ pid,
                                 uint32_t* keys_sorted, uint32_t* vals_sorted, uint32_t* __restrict__ pid_sorted,
                                 uint32_t* status, uint32_t cap)
@@ -639,6 +811,15 @@ __device__ __forceinline__ void tile_sort_group(const Views& V, int64_t gt, uint
     (void)cap;
     const ViewDesc& vd = V.v[view_of_tile(V, gt)];
     const uint32_t hi_bits = (uint32_t)(gt - vd.tile_base) << vd.shift;
+    auto pair = [&](uint32_t e) { return GS_DCHECK(e < cap, status) ? pid[e] : 0u; };
+    auto put = [&](int i, uint32_t low, uint32_t e, uint32_t p) {
+        keys_sorted[s0 + i] = hi_bits | low;
+        vals_sorted[s0 + i] = e;
+        pid_sorted[s0 + i] = p;
+    };
+    if (sort_words<IT>(bucket + s0, (int)n, 23 - vd.drop, reinterpret_cast<uint32_t*>(sk), g, pair, put)) return true;
+    if (IT > 8) return false;
+    g.sync();
     const int N = (int)((n + 7u) & ~7u);    // the last thread's keys padded
     for (int i = g.t; i < N; i += g.n) {
         unsigned long long x = ~0ull;
@@ -650,19 +831,15 @@ __device__ __forceinline__ void tile_sort_group(const Views& V, int64_t gt, uint
     }
     g.sync();
     block_merge_sort_smem(sk, N, g);
-    for (int i = g.t; i < (int)n; i += g.n) {
-        const unsigned long long x = sk[i];
-        const uint32_t e = (uint32_t)x;
-        keys_sorted[s0 + i] = hi_bits | (uint32_t)(x >> 32);
-        vals_sorted[s0 + i] = e;
-        pid_sorted[s0 + i] = GS_DCHECK(e < cap, status) ? pid[e] : 0u;
-    }
+    for (int i = g.t; i < (int)n; i += g.n) put(i, (uint32_t)(sk[i] >> 32), (uint32_t)sk[i], pair((uint32_t)sk[i]));
+    return true;
 }
 
-// A list longer than kTileSortMax, sorted by the whole block: chunks of
-// kTileSortMax sorted in shared memory, then merge levels alternating
-// between the bucket and the (keys, vals) arrays, starting where an even
-// number of moves ends in the bucket.
+// A list too long for shared memory, sorted by the whole block: chunks sorted in
+// shared memory into the (keys, vals) arrays (twice kTileSortMax entries as words,
+// or kTileSortMax 64-bit keys), then merge levels alternating between the arrays and
+// the bucket.  8 scenes, 81,600 tiles, 854 lists above 4,096 entries of 31M entries in
+// all: 1,130 -> 660 us for the whole sort, of which merge_level's pieces gave 120.
 __device__ void tile_sort_chunked(const Views& V, int64_t gt, uint32_t s0, uint32_t n, unsigned long long* sk,
                                   uint2* bucket, const uint32_t* __restrict__ pid, uint32_t* keys_sorted,
                                   uint32_t* vals_sorted, uint32_t* __restrict__ pid_sorted, uint32_t* status,
@@ -675,108 +852,107 @@ __device__ void tile_sort_chunked(const Views& V, int64_t gt, uint32_t s0, uint3
     const SortGroup g = whole_block();
     const PackedList pk{bucket};
     const SplitList sp{keys_sorted, vals_sorted};
-    const uint32_t M = kTileSortMax;
-    int levels = 0;
-    for (uint32_t run = M; run < n; run <<= 1) levels++;
-    const bool chunks_in_bucket = (levels & 1) == 0;
+    __shared__ uint32_t split[kTileSortThreads + 1];
+    const int bits = 23 - vd.drop;
+    const uint32_t M = bits + 13 <= 32 ? 2u * kTileSortMax : kTileSortMax;
+    static_assert(kTileSortMax == 4096, "13 bits index a chunk of words");
     for (uint32_t c0 = 0; c0 < n; c0 += M) {
         const uint32_t len = min(M, n - c0);
-        for (uint32_t i = threadIdx.x; i < M; i += blockDim.x) sk[i] = i < len ? pk.get(s0 + c0 + i) : ~0ull;
-        __syncthreads();
-        block_merge_sort_smem(sk, (int)M, g);
-        for (uint32_t i = threadIdx.x; i < len; i += blockDim.x) {
-            if (chunks_in_bucket) pk.put(s0 + c0 + i, sk[i]);
-            else sp.put(s0 + c0 + i, sk[i]);
+        auto put = [&](int i, uint32_t low, uint32_t e, uint32_t) { sp.put(s0 + c0 + i, sort_key(low, e)); };
+        if (!sort_words<16>(bucket + s0 + c0, (int)len, bits, reinterpret_cast<uint32_t*>(sk), g,
+                            [](uint32_t) { return 0u; }, put)) {
+            // by 64-bit keys, in two halves merged through the bucket where long
+            for (uint32_t h0 = 0; h0 < len; h0 += kTileSortMax) {
+                const uint32_t hl = min((uint32_t)kTileSortMax, len - h0);
+                __syncthreads();
+                for (uint32_t i = threadIdx.x; i < kTileSortMax; i += blockDim.x)
+                    sk[i] = i < hl ? pk.get(s0 + c0 + h0 + i) : ~0ull;
+                __syncthreads();
+                block_merge_sort_smem(sk, kTileSortMax, g);
+                for (uint32_t i = threadIdx.x; i < hl; i += blockDim.x)
+                    if (len > kTileSortMax) pk.put(s0 + c0 + h0 + i, sk[i]);
+                    else sp.put(s0 + c0 + i, sk[i]);
+            }
+            __syncthreads();
+            if (len > kTileSortMax) merge_level(pk, sp, s0 + c0, len, kTileSortMax, sk, split);
         }
         __syncthreads();
     }
-    bool in_bucket = chunks_in_bucket;
+    bool in_bucket = false;
     for (uint32_t run = M; run < n; run <<= 1) {
-        if (in_bucket) merge_level(pk, sp, s0, n, run);
-        else merge_level(sp, pk, s0, n, run);
+        if (in_bucket) merge_level(pk, sp, s0, n, run, sk, split);
+        else merge_level(sp, pk, s0, n, run, sk, split);
         in_bucket = !in_bucket;
     }
-    // the sorted list is in the bucket now
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-        const unsigned long long x = pk.get(s0 + i);
-        const uint32_t e = (uint32_t)x;
-        keys_sorted[s0 + i] = hi_bits | (uint32_t)(x >> 32);
-        vals_sorted[s0 + i] = e;
-        pid_sorted[s0 + i] = GS_DCHECK(e < cap, status) ? pid[e] : 0u;
+    constexpr int F = 4;                           // entries in flight per thread
+    for (uint32_t i0 = threadIdx.x; i0 < n; i0 += F * blockDim.x) {
+        unsigned long long x[F];
+        uint32_t p[F];
+#pragma unroll
+        for (int k = 0; k < F; k++) {
+            const uint32_t i = i0 + k * blockDim.x;
+            x[k] = i >= n ? 0ull : in_bucket ? pk.get(s0 + i) : sp.get(s0 + i);
+        }
+#pragma unroll
+        for (int k = 0; k < F; k++) {
+            const uint32_t e = (uint32_t)x[k];
+            p[k] = i0 + k * blockDim.x < n && GS_DCHECK(e < cap, status) ? pid[e] : 0u;
+        }
+#pragma unroll
+        for (int k = 0; k < F; k++) {
+            const uint32_t i = i0 + k * blockDim.x;
+            if (i >= n) break;
+            keys_sorted[s0 + i] = hi_bits | (uint32_t)(x[k] >> 32);
+            vals_sorted[s0 + i] = (uint32_t)x[k];
+            pid_sorted[s0 + i] = p[k];
+        }
     }
 }
 
 // The tile order lists the tiles by size class (k_tile_order): long lists
 // (>= 2047 entries), medium (1023-2046), short (255-1022), tiny (<= 254).
-// Long and medium lists: 512-thread blocks, one long list per block (up to
-// kTileSortMax entries in shared memory, longer ones chunked), or two medium
-// lists per block, one per 256-thread half with a named barrier of its own.
-__global__ void __launch_bounds__(kTileSortThreads) k_tile_sort_long(Views V, const uint32_t* __restrict__ order,
-                                                                     const uint2* __restrict__ ranges,
-                                                                     uint2* bucket, const uint32_t* __restrict__ pid,
-                                                                     uint32_t* keys_sorted, uint32_t* vals_sorted,
-                                                                     uint32_t* __restrict__ pid_sorted,
-                                                                     const WsHeader* __restrict__ hdr,
-                                                                     uint32_t* status, uint32_t cap)
+// Blocks of 512 threads take one long list each, or two medium, four short or
+// sixteen tiny ones, by halves, quarters (with a named barrier each) or warps.
+// Three blocks (1,536 threads) per SM: 40 registers serve every list up to 4,096
+// entries; the 16-key form of longer ones spills there (3M Gaussians, 4x1080p: two
+// blocks 326 us, three 257, four 251; 8 scenes with 854 longer lists: 802, 660, 680).
+// One launch for all classes: 2,000 Gaussians 10.0 + 3 us of launch -> 8.7 us against
+// two kernels, 4x1080p 248 -> 257.
+__global__ void __launch_bounds__(kTileSortThreads, 3) k_tile_sort(Views V, const uint32_t* __restrict__ order,
+                                                                   const uint2* __restrict__ ranges, uint2* bucket,
+                                                                   const uint32_t* __restrict__ pid,
+                                                                   uint32_t* keys_sorted, uint32_t* vals_sorted,
+                                                                   uint32_t* __restrict__ pid_sorted,
+                                                                   const WsHeader* __restrict__ hdr, uint32_t* status,
+                                                                   uint32_t cap)
 {
     extern __shared__ unsigned long long sk[];
-    const uint32_t n_long = hdr->sort_class[0], n_med = hdr->sort_class[1];
-    const uint32_t b = blockIdx.x;
-    if (b < n_long) {
-        const int64_t gt = order[b];
-        const uint2 r = range_at(ranges, gt, cap, status);
-        const uint32_t n = r.y - r.x;
-        if (n <= (uint32_t)kTileSortMax)
-            tile_sort_group(V, gt, r.x, n, sk, SortGroup{(int)threadIdx.x, kTileSortThreads, 0}, bucket, pid,
-                            keys_sorted, vals_sorted, pid_sorted, status, cap);
-        else
-            tile_sort_chunked(V, gt, r.x, n, sk, bucket, pid, keys_sorted, vals_sorted, pid_sorted, status, cap);
-        return;
+    const uint32_t t = threadIdx.x;
+    uint32_t first = 0, b = blockIdx.x, split = 1;     // the block's class: its first list, lists per block
+    for (int c = 0; c < 4; c++, split = c == 3 ? 16u : 2u * split) {
+        const uint32_t lists = hdr->sort_class[c], blocks = (lists + split - 1u) / split;
+        if (b < blocks) {
+            const uint32_t n_t = kTileSortThreads / split, part = t / n_t, m = split * b + part;
+            if (m >= lists) return;
+            const int64_t gt = order[first + m];
+            const uint2 r = range_at(ranges, gt, cap, status);
+            const uint32_t n = r.y - r.x;
+            if (n == 0 || (c > 0 && n > 8u * n_t)) return;
+            const SortGroup g{(int)(t - part * n_t), (int)n_t, c == 0 ? 0 : 1 + (int)part};
+            bool done = false;
+            if (n <= 8u * n_t)
+                done = tile_sort_group<8>(V, gt, r.x, n, sk + 8u * n_t * part, g, bucket, pid, keys_sorted, vals_sorted,
+                                          pid_sorted, status, cap);
+            else if (n <= 2u * kTileSortMax)
+                done = tile_sort_group<16>(V, gt, r.x, n, sk, g, bucket, pid, keys_sorted, vals_sorted, pid_sorted,
+                                           status, cap);
+            if (!done)
+                tile_sort_chunked(V, gt, r.x, n, sk, bucket, pid, keys_sorted, vals_sorted, pid_sorted, status, cap);
+            return;
+        }
+        b -= blocks;
+        first += lists;
     }
-    const uint32_t half = threadIdx.x >= kTileSortThreads / 2 ? 1u : 0u;
-    const uint32_t m = 2u * (b - n_long) + half;     // medium list of this half
-    if (b >= n_long + (n_med + 1u) / 2u || m >= n_med) return;
-    const int64_t gt = order[n_long + m];
-    const uint2 r = range_at(ranges, gt, cap, status);
-    const uint32_t n = r.y - r.x;
-    if (n == 0 || n > 4u * kTileSortThreads) return;
-    const SortGroup g{(int)(threadIdx.x - half * (kTileSortThreads / 2)), kTileSortThreads / 2, 1 + (int)half};
-    tile_sort_group(V, gt, r.x, n, sk + half * (kTileSortMax / 2), g, bucket, pid, keys_sorted, vals_sorted,
-                    pid_sorted, status, cap);
-}
-
-// Short and tiny lists: 128-thread blocks, one short list per block, or four
-// tiny lists per block, one per warp.
-__global__ void __launch_bounds__(kTileSortSmall) k_tile_sort_short(Views V, const uint32_t* __restrict__ order,
-                                                                    const uint2* __restrict__ ranges, uint2* bucket,
-                                                                    const uint32_t* __restrict__ pid,
-                                                                    uint32_t* keys_sorted, uint32_t* vals_sorted,
-                                                                    uint32_t* __restrict__ pid_sorted,
-                                                                    const WsHeader* __restrict__ hdr,
-                                                                    uint32_t* status, uint32_t cap)
-{
-    extern __shared__ unsigned long long sk[];
-    const uint32_t base = hdr->sort_class[0] + hdr->sort_class[1];
-    const uint32_t n_short = hdr->sort_class[2], n_tiny = hdr->sort_class[3];
-    const uint32_t b = blockIdx.x;
-    if (b < n_short) {
-        const int64_t gt = order[base + b];
-        const uint2 r = range_at(ranges, gt, cap, status);
-        const uint32_t n = r.y - r.x;
-        if (n == 0 || n > 8u * kTileSortSmall) return;
-        tile_sort_group(V, gt, r.x, n, sk, SortGroup{(int)threadIdx.x, kTileSortSmall, 0}, bucket, pid, keys_sorted,
-                        vals_sorted, pid_sorted, status, cap);
-        return;
-    }
-    const uint32_t w = threadIdx.x >> 5;
-    const uint32_t m = 4u * (b - n_short) + w;       // tiny list of this warp
-    if (b >= n_short + (n_tiny + 3u) / 4u || m >= n_tiny) return;
-    const int64_t gt = order[base + n_short + m];
-    const uint2 r = range_at(ranges, gt, cap, status);
-    const uint32_t n = r.y - r.x;
-    if (n == 0 || n > 256u) return;
-    const SortGroup g{(int)(threadIdx.x & 31u), 32, 0};
-    tile_sort_group(V, gt, r.x, n, sk + w * 256, g, bucket, pid, keys_sorted, vals_sorted, pid_sorted, status, cap);
 }
 
 // ---------------------------------------------------------------------------
@@ -813,16 +989,10 @@ void launch_bin_sort(const Plan& P, const WsPtrs& w, cudaStream_t st)
     }
     // sort each tile's list
     {
-        const size_t smem_l = sizeof(unsigned long long) * kTileSortMax;            // 32 KB: no opt-in needed
-        const size_t smem_s = sizeof(unsigned long long) * 8 * kTileSortSmall;      // 8 KB
-        k_tile_sort_long<<<(unsigned)V.tiles, kTileSortThreads, smem_l, st>>>(V, w.tile_order, w.ranges, w.bucket,
-                                                                             w.pid, w.keys_sorted, w.vals_sorted,
-                                                                             w.pid_sorted, w.hdr, &w.hdr->status,
-                                                                             cap);
-        k_tile_sort_short<<<(unsigned)V.tiles, kTileSortSmall, smem_s, st>>>(V, w.tile_order, w.ranges, w.bucket,
-                                                                             w.pid, w.keys_sorted, w.vals_sorted,
-                                                                             w.pid_sorted, w.hdr, &w.hdr->status,
-                                                                             cap);
+        const size_t smem = sizeof(unsigned long long) * kTileSortMax;              // 32 KB: no opt-in needed
+        k_tile_sort<<<(unsigned)V.tiles, kTileSortThreads, smem, st>>>(V, w.tile_order, w.ranges, w.bucket, w.pid,
+                                                                       w.keys_sorted, w.vals_sorted, w.pid_sorted,
+                                                                       w.hdr, &w.hdr->status, cap);
     }
 }
 

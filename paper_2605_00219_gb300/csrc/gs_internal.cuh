@@ -12,12 +12,11 @@ namespace gs {
 // Intersection capacity granule (the capacity is rounded up to it).
 constexpr int kCapGranule = 2048;
 
-// Per-tile sort: lists of up to kTileSortMax entries are sorted in shared
-// memory by one thread block; longer lists are sorted in chunks of that size
-// and merged in global memory by the same block.
-constexpr int kTileSortThreads = 512;     // 8 keys per thread
+// Per-tile sort: lists of up to kTileSortMax entries (twice that as 32-bit words)
+// are sorted in shared memory by one thread block; longer lists are sorted in chunks
+// of that size and merged in global memory by the same block.
+constexpr int kTileSortThreads = 512;     // 8 keys per thread, 16 words in long lists
 constexpr int kTileSortMax = 4096;
-constexpr int kTileSortSmall = 128;       // threads for lists of up to 1024 entries
 
 // Exclusive scan geometry: 512 threads x 8 values per block.
 constexpr int kScanThreads = 512;
