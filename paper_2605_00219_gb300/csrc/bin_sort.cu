@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(1024) k_sort_setup(const uint32_t* __restrict_
                                                      uint32_t* __restrict__ total_at, WsHeader* __restrict__ hdr,
                                                      uint32_t cap)
 {
+    if (!after_previous()) return;
     constexpr int IT = kScanBlock / 1024;
     __shared__ unsigned long long ws64[32];
     __shared__ uint32_t ws[32], hist[32];
@@ -215,6 +216,7 @@ __global__ void __launch_bounds__(kScanThreads) k_sort_sums(const uint32_t* __re
                                                             const uint32_t* __restrict__ cnt,
                                                             uint32_t* __restrict__ part)
 {
+    if (!after_previous()) return;
     __shared__ uint32_t ws[32], hist[32];
     if (blockIdx.x < gblocks16) {
         const int64_t g = (int64_t)blockIdx.x * (kScanThreads / 32) + (threadIdx.x >> 5);
@@ -251,6 +253,7 @@ __global__ void __launch_bounds__(1024) k_sort_parts(uint32_t* __restrict__ gpar
                                                      uint32_t* __restrict__ total_at, WsHeader* __restrict__ hdr,
                                                      uint32_t cap)
 {
+    if (!after_previous()) return;
     __shared__ unsigned long long ws64[32];
     __shared__ uint32_t ws[32], place[32];
     const bool fits = scan_gpart(gpart, gblocks, hdr, total_at, cap, ws64);
@@ -292,6 +295,7 @@ __global__ void __launch_bounds__(kScanThreads) k_tile_down(int64_t tiles, uint3
                                                             uint2* __restrict__ ranges, uint32_t* __restrict__ order,
                                                             const WsHeader* __restrict__ hdr)
 {
+    if (!after_previous()) return;
     __shared__ uint32_t ws[32], hist[32];
     __shared__ uint32_t buf[kScanBlock];
     const int64_t base = (int64_t)blockIdx.x * kScanBlock;
@@ -362,6 +366,7 @@ __global__ void __launch_bounds__(kEmitThreads, 5) k_emit(Views V, const uint32_
                                                  uint2* __restrict__ bucket, uint32_t* __restrict__ pid,
                                                  WsHeader* __restrict__ hdr)
 {
+    if (!after_previous()) return;
     __shared__ uint32_t ws[32], earlier[kEmitThreads / 32];
     const int64_t qb = (int64_t)blockIdx.x * kEmitThreads, qi = qb + threadIdx.x;
     // the pair's loads are issued together, before any of them is tested
@@ -926,6 +931,7 @@ __global__ void __launch_bounds__(kTileSortThreads, 3) k_tile_sort(Views V, cons
                                                                    const WsHeader* __restrict__ hdr, uint32_t* status,
                                                                    uint32_t cap)
 {
+    if (!after_previous()) return;
     extern __shared__ unsigned long long sk[];
     const uint32_t t = threadIdx.x;
     uint32_t first = 0, b = blockIdx.x, split = 1;     // the block's class: its first list, lists per block
@@ -969,28 +975,28 @@ void launch_bin_sort(const Plan& P, const WsPtrs& w, cudaStream_t st)
     const unsigned nparts = one ? 0u : (unsigned)P.tile_scan_parts;
     if (sums) {
         const unsigned gb = (unsigned)((P.pair_groups + kScanThreads / 32 - 1) / (kScanThreads / 32));
-        k_sort_sums<<<gb + nparts, kScanThreads, 0, st>>>(w.count, V.pairs, w.gpart, P.pair_groups, gb, V.tiles,
+        launch_after(k_sort_sums, gb + nparts, kScanThreads, 0, st, w.count, V.pairs, w.gpart, P.pair_groups, gb, V.tiles,
                                                           w.tile_cnt, w.tile_part);
     }
     if (one) {
-        k_sort_setup<<<1, 1024, 0, st>>>(w.count, V.pairs, sums, w.gpart, P.pair_groups, (int)V.tiles, w.tile_cnt,
+        launch_after(k_sort_setup, 1, 1024, 0, st, w.count, V.pairs, sums, w.gpart, P.pair_groups, (int)V.tiles, w.tile_cnt,
                                          w.tile_cur, w.ranges, w.tile_order, total_at, w.hdr, cap);
     } else {
-        k_sort_parts<<<1, 1024, 0, st>>>(w.gpart, P.pair_groups, V.tiles, w.tile_part, nparts, total_at, w.hdr, cap);
-        k_tile_down<<<nparts, kScanThreads, 0, st>>>(V.tiles, w.tile_cnt, w.tile_part, w.tile_cur, w.ranges,
+        launch_after(k_sort_parts, 1, 1024, 0, st, w.gpart, P.pair_groups, V.tiles, w.tile_part, nparts, total_at, w.hdr, cap);
+        launch_after(k_tile_down, nparts, kScanThreads, 0, st, V.tiles, w.tile_cnt, w.tile_part, w.tile_cur, w.ranges,
                                                      w.tile_order, w.hdr);
     }
     // generate keys into the tile buckets
     {
         const int64_t blocks = (V.pairs + kEmitThreads - 1) / kEmitThreads;
-        k_emit<<<(unsigned)blocks, kEmitThreads, 0, st>>>(V, w.count, w.gpart, w.offset, w.rec, w.span, w.rank,
+        launch_after(k_emit, (unsigned)blocks, kEmitThreads, 0, st, V, w.count, w.gpart, w.offset, w.rec, w.span, w.rank,
                                                           w.tile_cur, w.tile_cnt + V.tiles, w.bucket, w.pid,
                                                           w.hdr);
     }
     // sort each tile's list
     {
         const size_t smem = sizeof(unsigned long long) * kTileSortMax;              // 32 KB: no opt-in needed
-        k_tile_sort<<<(unsigned)V.tiles, kTileSortThreads, smem, st>>>(V, w.tile_order, w.ranges, w.bucket, w.pid,
+        launch_after(k_tile_sort, (unsigned)V.tiles, kTileSortThreads, smem, st, V, w.tile_order, w.ranges, w.bucket, w.pid,
                                                                        w.keys_sorted, w.vals_sorted, w.pid_sorted,
                                                                        w.hdr, &w.hdr->status, cap);
     }

@@ -201,6 +201,7 @@ Scenes make_scenes(const Plan& P, const gs_scene_buf* scenes)
 // counters that the projection adds to start from zero.
 __global__ void k_ws_init(WsHeader* hdr, int full, uint32_t* __restrict__ tile_cnt, int64_t n_cnt)
 {
+    if (!after_previous()) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         hdr->status = 0;
         hdr->k_required = 0;
@@ -221,20 +222,21 @@ static unsigned init_blocks(const Plan& P)
 
 void launch_ws_init(const Plan& P, const WsPtrs& w, cudaStream_t st)
 {
-    k_ws_init<<<init_blocks(P), 256, 0, st>>>(w.hdr, 1, w.tile_cnt, 2 * P.views.tiles);
+    launch_after(k_ws_init, init_blocks(P), 256, 0, st, w.hdr, 1, w.tile_cnt, 2 * P.views.tiles);
 }
 
 static void launch_step_begin(const Plan& P, const WsPtrs& w, cudaStream_t st)
 {
-    k_ws_init<<<init_blocks(P), 256, 0, st>>>(w.hdr, 0, w.tile_cnt, 2 * P.views.tiles);
+    launch_after(k_ws_init, init_blocks(P), 256, 0, st, w.hdr, 0, w.tile_cnt, 2 * P.views.tiles);
 }
 
 __global__ void k_adam_advance(WsHeader* hdr)
 {
+    if (!after_previous()) return;
     if (threadIdx.x == 0) hdr->step += 1;
 }
 
-void launch_adam_advance(const WsPtrs& w, cudaStream_t st) { k_adam_advance<<<1, 32, 0, st>>>(w.hdr); }
+void launch_adam_advance(const WsPtrs& w, cudaStream_t st) { launch_after(k_adam_advance, 1, 32, 0, st, w.hdr); }
 
 __global__ void k_set_step(WsHeader* hdr, int32_t step)
 {

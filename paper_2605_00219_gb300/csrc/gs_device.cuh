@@ -9,6 +9,23 @@
 
 namespace gs {
 
+// Every kernel of a step starts with `if (!after_previous()) return;` and is launched
+// by launch_after: its blocks may be scheduled while the last blocks of the previous
+// kernel of the stream still run, wait here for that kernel's end and its writes, and
+// then let the next kernel do the same (after the wait, so that at most two kernels
+// are resident).  Always true (the grid is not empty), which the compiler cannot know:
+// no load, also none marked read-only, can be moved from behind the branch to before
+// the wait.
+__device__ __forceinline__ bool after_previous()
+{
+    uint32_t grid;
+    asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;\n\tmov.u32 %0, %%nctaid.x;"
+                 : "=r"(grid)
+                 :
+                 : "memory");
+    return grid != 0u;
+}
+
 constexpr int kMaxViews = GS_MAX_VIEWS;
 constexpr int kMaxScenes = GS_MAX_SCENES;
 

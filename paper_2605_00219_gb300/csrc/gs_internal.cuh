@@ -4,10 +4,35 @@
 #include <algorithm>
 #include <cstddef>
 #include <cstring>
+#include <utility>
 
 #include "gs_device.cuh"
 
 namespace gs {
+
+// Launch of a kernel that starts with after_previous(): programmatic dependent launch,
+// which hides the launch of a kernel behind the end of the one before it in the stream
+// (2,000 Gaussians, eleven launches: 94 -> 72 us a step; 200k, 720p: a render 153 -> 143
+// us).  Not under capture: a graph's plain edges cost less than the waiting blocks do
+// (200k, 720p step 313 against 325 us; 3M, 4x1080p 6.00 against 6.08 ms; only the
+// smallest graph gains, 71.8 -> 70.1 us).
+template <typename... Params, typename... Args>
+inline void launch_after(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(st, &capture);
+    cfg.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
 
 // Intersection capacity granule (the capacity is rounded up to it).
 constexpr int kCapGranule = 2048;

@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(kSsThreads, 3) k_loss_l1_ssim(Views V, const f
                                                                 float inv_n, float* __restrict__ dl,
                                                                 float* __restrict__ part, WsHeader* __restrict__ hdr)
 {
+    if (!after_previous()) return;
     extern __shared__ __align__(16) unsigned char ssim_smem[];
     SsimSmem& sm = *reinterpret_cast<SsimSmem*>(ssim_smem);
     __shared__ float red[2][kSsThreads / 32];
@@ -396,7 +397,7 @@ void launch_loss_l1_ssim(const Plan& P, const WsPtrs& w, const float* image, con
     do {                                                                                                            \
         cudaFuncSetAttribute(k_loss_l1_ssim<MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize,                     \
                              (int)sizeof(SsimSmem));                                                                \
-        k_loss_l1_ssim<MASK><<<(unsigned)blocks, kSsThreads, sizeof(SsimSmem), st>>>(P.views, image, t, lam, inv_n, \
+        launch_after(k_loss_l1_ssim<MASK>, (unsigned)blocks, kSsThreads, sizeof(SsimSmem), st, P.views, image, t, lam, inv_n, \
                                                                                     dl, w.loss_part, w.hdr);       \
     } while (0)
     if (alpha_mask) GS_SSIM(true);

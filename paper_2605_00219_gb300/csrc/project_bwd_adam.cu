@@ -375,6 +375,7 @@ __global__ void __launch_bounds__(kPbaThreads, 4) k_project_bwd_adam(Views V, Sc
                                                                   float4* __restrict__ grads_out,
                                                                   const WsHeader* __restrict__ hdr, uint32_t cap)
 {
+    if (!after_previous()) return;
     // per thread, a row of 12 float4 (stride 13 float4: the 16-byte accesses
     // of 8 consecutive threads cover all 32 banks once) for the SH gradients,
     // and a row of the Gaussian's 48 SH coefficients as stored (FP32 or BF16,
@@ -640,7 +641,7 @@ void launch_project_bwd_adam(const Plan& P, const Scenes& S, const float* cams, 
         /* 53 KB (FP32 rows) or 41 KB: above the default 48 KB for FP32 */                                          \
         const size_t smem = (sizeof(float4) * 13 + ShRow<SH>::kRowBytes) * kPbaThreads;                              \
         cudaFuncSetAttribute(k_project_bwd_adam<SH, MO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);   \
-        k_project_bwd_adam<SH, MO><<<(unsigned)blocks, kPbaThreads, smem, st>>>(P.views, S, cams, w.count, w.offset, \
+        launch_after(k_project_bwd_adam<SH, MO>, (unsigned)blocks, kPbaThreads, smem, st, P.views, S, cams, w.count, w.offset, \
                               w.gradrec, A, reinterpret_cast<float4*>(grads_out), w.hdr, (uint32_t)P.cap);         \
     } while (0)
     if (!P.sh_bf16 && !P.mom_bf16) GS_PBA(false, false);

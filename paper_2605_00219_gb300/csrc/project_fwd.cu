@@ -136,6 +136,7 @@ __global__ void __launch_bounds__(256, 4) k_project_fwd(Views V, Scenes S, const
                                                      uint4* __restrict__ rank,
                                                      WsHeader* __restrict__ hdr)
 {
+    if (!after_previous()) return;
     // the views' field-of-view limits, once per block (two correctly
     // rounded divisions a view instead of a pair)
     __shared__ float2 slim[kMaxViews];
@@ -178,7 +179,7 @@ void launch_project_fwd(const Plan& P, const Scenes& S, const float* cams, const
     const int T = 256;
     const int64_t blocks = (S.total + T - 1) / T;
     if (blocks == 0) return;
-    k_project_fwd<<<(unsigned)blocks, T, 0, st>>>(P.views, S, cams, w.count, w.tile_cnt, w.rec, w.span, w.rank, w.hdr);
+    launch_after(k_project_fwd, (unsigned)blocks, T, 0, st, P.views, S, cams, w.count, w.tile_cnt, w.rec, w.span, w.rank, w.hdr);
 }
 
 }  // namespace gs

@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_raster_bwd(Views V, const uint3
                                                             const uint32_t* __restrict__ nlast,
                                                             GradRec* __restrict__ gradrec, int fixed_S)
 {
+    if (!after_previous()) return;
     extern __shared__ float4 smem4[];
     BwdSmem sm;
     sm.runA = smem4;
@@ -382,6 +383,7 @@ k_raster_bwd_blocks(Views V, const uint32_t* __restrict__ order, const uint2* __
                     const float* __restrict__ dl, const uint32_t* __restrict__ nlast, GradRec* __restrict__ gradrec,
                     uint32_t* __restrict__ status, uint32_t cap)
 {
+    if (!after_previous()) return;
     using B = BwdBlocks<TW, TH, GL>;
     constexpr int NT = B::kThreads, NC = B::kCols, NB = B::kBlocks, BB = B::kBatch, S = B::kSlots;
     constexpr int NG = B::kGroups;
@@ -739,7 +741,7 @@ void launch_raster_bwd(const Plan& P, const WsPtrs& w, const float* image, const
             cudaFuncSetAttribute(k_raster_bwd<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb);   \
             attr_set = true;                                                                                \
         }                                                                                                   \
-        k_raster_bwd<NP><<<grid, kBwdThreads, sb, st>>>(V, w.tile_order, w.ranges, w.vals_sorted, w.pid_sorted, w.rec, image, \
+        launch_after(k_raster_bwd<NP>, grid, kBwdThreads, sb, st, V, w.tile_order, w.ranges, w.vals_sorted, w.pid_sorted, w.rec, image, \
                                                         dl, w.nlast, w.gradrec, fixed);                     \
     } while (0)
     if (np == 64) GS_RB(64);
@@ -831,6 +833,7 @@ __global__ void __launch_bounds__(BS) k_raster_bwd_px(Views V, const uint32_t* _
                                                       GradRec* __restrict__ gradrec, uint32_t* __restrict__ status,
                                                       uint32_t cap)
 {
+    if (!after_previous()) return;
     constexpr int NW = BS / 32;
     constexpr int BH = 4 * PPT;            // warp block height, pixels
     constexpr int TH = BS * PPT / TW;      // tile height, pixels
@@ -1055,11 +1058,11 @@ void launch_raster_bwd_px(const Plan& P, const WsPtrs& w, const float* bg, const
     const unsigned grid = (unsigned)V.tiles;
     const int ppt = tile_ppt(P);
 #define GS_RBP(BS, TW, PPT)                                                                                  \
-    k_raster_bwd_px<BS, TW, PPT><<<grid, BS, 0, st>>>(V, w.tile_order, w.ranges, w.vals_sorted, w.pid_sorted, \
+    launch_after(k_raster_bwd_px<BS, TW, PPT>, grid, BS, 0, st, V, w.tile_order, w.ranges, w.vals_sorted, w.pid_sorted, \
                                                       w.rec, w.tfinal, bg, dl, w.nlast, w.gradrec, &w.hdr->status,   \
                                                       (uint32_t)P.cap)
 #define GS_RBB(TW, TH, GL)                                                                                    \
-    k_raster_bwd_blocks<TW, TH, GL><<<grid, BwdBlocks<TW, TH, GL>::kThreads, 0, st>>>(                         \
+    launch_after(k_raster_bwd_blocks<TW, TH, GL>, grid, BwdBlocks<TW, TH, GL>::kThreads, 0, st,                          \
         V, w.tile_order, w.ranges, w.vals_sorted, w.pid_sorted, w.rec, w.tfinal, bg, dl, w.nlast, w.gradrec,   \
         &w.hdr->status, (uint32_t)P.cap)
     // 16-wide tiles with one pixel per thread (the default) walk 8x4 blocks,

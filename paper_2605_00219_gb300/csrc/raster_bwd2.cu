@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(BS) k_raster_bwd2(Views V, const uint32_t* __r
                                                     const uint32_t* __restrict__ nlast,
                                                     GradRec* __restrict__ gradrec)
 {
+    if (!after_previous()) return;
     using C = Bwd2Cfg<BS>;
     constexpr int NW = C::NW, BB = C::BB, NP = C::NP, NPS = C::NPS, TPP = C::TPP, PPT = C::PPT;
     constexpr int WPR = TW / 8;            // 8x4 warp blocks per tile row
@@ -331,7 +332,7 @@ void launch_raster_bwd2(const Plan& P, const WsPtrs& w, const float* bg, const f
             cudaFuncSetAttribute(k_raster_bwd2<BS, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb); \
             attr_set = true;                                                                                  \
         }                                                                                                     \
-        k_raster_bwd2<BS, TW><<<grid, BS, sb, st>>>(V, w.tile_order, w.ranges, w.vals_sorted, w.pid_sorted, w.rec, w.tfinal, \
+        launch_after(k_raster_bwd2<BS, TW>, grid, BS, sb, st, V, w.tile_order, w.ranges, w.vals_sorted, w.pid_sorted, w.rec, w.tfinal, \
                                                      bg, dl, w.nlast, w.gradrec);                             \
     } while (0)
     if (V.tw == 8) GS_RB2(64, 8);

@@ -30,6 +30,7 @@ k_raster_fwd(Views V, const uint32_t* __restrict__ order, const uint2* __restric
              float* __restrict__ image, float* __restrict__ tfinal, uint32_t* __restrict__ nlast,
              WsHeader* __restrict__ hdr, uint32_t cap)
 {
+    if (!after_previous()) return;
     using TB = TileBlocks<TW, TH>;
     constexpr int NT = TB::kThreads, NW = TB::kWarps, CH = TW == 8 ? 64 : 128;   // CH: list entries per staged chunk
     constexpr int IPT = (CH + NT - 1) / NT;      // staged entries per thread
@@ -218,7 +219,7 @@ void launch_raster_fwd(const Plan& P, const WsPtrs& w, const float* bg, float* i
 {
     const Views& V = P.views;
     const unsigned grid = (unsigned)V.tiles;
-#define GS_RF(TW, TH) k_raster_fwd<TW, TH><<<grid, TileBlocks<TW, TH>::kThreads, 0, st>>>(                          \
+#define GS_RF(TW, TH) launch_after(k_raster_fwd<TW, TH>, grid, TileBlocks<TW, TH>::kThreads, 0, st,                           \
         V, w.tile_order, w.ranges, w.pid_sorted, w.rec, bg, image, w.tfinal, w.nlast, w.hdr, (uint32_t)P.cap)
     if (V.tw == 8) GS_RF(8, 8);
     else if (V.th == 16) GS_RF(16, 16);
@@ -244,6 +245,7 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_l1(const float* __restric
                                                           int64_t n, float inv_n, float* __restrict__ part,
                                                           WsHeader* __restrict__ hdr)
 {
+    if (!after_previous()) return;
     __shared__ float ws[kLossThreads / 32];
     __shared__ bool is_last;
     float s = 0.f;
@@ -325,10 +327,10 @@ void launch_loss_l1(const Plan& P, const WsPtrs& w, const float* image, const fl
     const int64_t per_block = (int64_t)kLossThreads * kLossItems * (vec ? 2 : 1);
     const int64_t blocks = (n + per_block - 1) / per_block;
     if (vec)
-        k_loss_l1<true><<<(unsigned)blocks, kLossThreads, 0, st>>>(image, target, dl, n, 1.0f / (float)n,
+        launch_after(k_loss_l1<true>, (unsigned)blocks, kLossThreads, 0, st, image, target, dl, n, 1.0f / (float)n,
                                                                    w.loss_part, w.hdr);
     else
-        k_loss_l1<false><<<(unsigned)blocks, kLossThreads, 0, st>>>(image, target, dl, n, 1.0f / (float)n,
+        launch_after(k_loss_l1<false>, (unsigned)blocks, kLossThreads, 0, st, image, target, dl, n, 1.0f / (float)n,
                                                                     w.loss_part, w.hdr);
 }
 
