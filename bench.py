@@ -568,7 +568,7 @@ def main():
                        "views_per_step": nviews},
             "e2e": {"value": ws * nviews * 1e3 / e2e_ms, "unit": "view-steps/s", "h2d_bytes_per_step": int(h2d),
                     "d2h_bytes_per_step": d2h},
-            "gpu_launches": int(args.steps * launches_per_step(tr.plan)),
+            "gpu_launches": int(args.steps * step_kernels(tr.plan)),
             "roofline": roof,
             "rooflines": rooflines,
             "plain_fp32": None if plain_ms is None else {
@@ -678,12 +678,23 @@ def stage_rooflines(work, stage_ms, hbm_peak_gbs, alu_peak_tflops):
 
 
 def launches_per_step(plan) -> int:
-    """Kernels of this library launched by one step (see the launchers)."""
+    """Kernels of a step whose sort takes ten launches, the count of the first
+    recorded launch list; step_kernels is what a plan launches now."""
     project = 2                                        # header reset + projection
-    binsort = 3 + 3 + 1 + 1 + 2                        # count scan (with K and the capacity check), tile scan
-                                                       # (with the ranges), order, emit, sort (long and short
-                                                       # lists)
+    binsort = 3 + 3 + 1 + 1 + 2                        # count scan, tile scan, order, emission, two sorts
     return project + binsort + 1 + 1 + 1 + 1 + 1       # raster fwd, loss, raster bwd, proj bwd+adam, advance
+
+
+def step_kernels(plan) -> int:
+    """Kernels of this library launched by one step (see the launchers).  The
+    set-up of the sort is one block up to 4,096 tiles, which also sums the pairs
+    up to 64 groups of 1,024, and three launches above."""
+    project = 2                                        # header reset + projection
+    if plan.tiles > 4096:
+        setup = 3                                      # sums, parts, tile starts
+    else:
+        setup = 1 + int(-(-plan.pairs // 1024) > 64)
+    return project + setup + 1 + 1 + 1 + 1 + 1 + 1 + 1   # emit, sort, raster fwd, loss, raster bwd, adam, advance
 
 
 if __name__ == "__main__":

@@ -5,8 +5,8 @@ rasterization-backward implementations, Sec. 4.2).
 
 A candidate is (tile, bwd_impl, threads_per_tile).  The pixel-parallel
 backward (impl 0) runs with one, two or (16-wide tiles) four pixels per
-thread; the other two backward implementations, and the raster forward, with
-one thread per pixel.
+thread; the other two backward implementations have one thread per pixel, and
+the raster forward one shape per tile size.
 
 Each candidate keeps a Normal-Inverse-Gamma posterior over its latency.  A
 round samples one latency per candidate from its posterior, runs the

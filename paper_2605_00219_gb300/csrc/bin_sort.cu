@@ -914,7 +914,7 @@ __device__ void tile_sort_chunked(const Views& V, int64_t gt, uint32_t s0, uint3
     }
 }
 
-// The tile order lists the tiles by size class (k_tile_order): long lists
+// The tile order lists the tiles by size class (see len_bucket): long lists
 // (>= 2047 entries), medium (1023-2046), short (255-1022), tiny (<= 254).
 // Blocks of 512 threads take one long list each, or two medium, four short or
 // sixteen tiny ones, by halves, quarters (with a named barrier each) or warps.
@@ -975,30 +975,29 @@ void launch_bin_sort(const Plan& P, const WsPtrs& w, cudaStream_t st)
     const unsigned nparts = one ? 0u : (unsigned)P.tile_scan_parts;
     if (sums) {
         const unsigned gb = (unsigned)((P.pair_groups + kScanThreads / 32 - 1) / (kScanThreads / 32));
-        launch_after(k_sort_sums, gb + nparts, kScanThreads, 0, st, w.count, V.pairs, w.gpart, P.pair_groups, gb, V.tiles,
-                                                          w.tile_cnt, w.tile_part);
+        launch_after(k_sort_sums, gb + nparts, kScanThreads, 0, st, w.count, V.pairs, w.gpart, P.pair_groups, gb,
+                     V.tiles, w.tile_cnt, w.tile_part);
     }
     if (one) {
-        launch_after(k_sort_setup, 1, 1024, 0, st, w.count, V.pairs, sums, w.gpart, P.pair_groups, (int)V.tiles, w.tile_cnt,
-                                         w.tile_cur, w.ranges, w.tile_order, total_at, w.hdr, cap);
+        launch_after(k_sort_setup, 1, 1024, 0, st, w.count, V.pairs, sums, w.gpart, P.pair_groups, (int)V.tiles,
+                     w.tile_cnt, w.tile_cur, w.ranges, w.tile_order, total_at, w.hdr, cap);
     } else {
-        launch_after(k_sort_parts, 1, 1024, 0, st, w.gpart, P.pair_groups, V.tiles, w.tile_part, nparts, total_at, w.hdr, cap);
+        launch_after(k_sort_parts, 1, 1024, 0, st, w.gpart, P.pair_groups, V.tiles, w.tile_part, nparts, total_at,
+                     w.hdr, cap);
         launch_after(k_tile_down, nparts, kScanThreads, 0, st, V.tiles, w.tile_cnt, w.tile_part, w.tile_cur, w.ranges,
-                                                     w.tile_order, w.hdr);
+                     w.tile_order, w.hdr);
     }
     // generate keys into the tile buckets
     {
         const int64_t blocks = (V.pairs + kEmitThreads - 1) / kEmitThreads;
-        launch_after(k_emit, (unsigned)blocks, kEmitThreads, 0, st, V, w.count, w.gpart, w.offset, w.rec, w.span, w.rank,
-                                                          w.tile_cur, w.tile_cnt + V.tiles, w.bucket, w.pid,
-                                                          w.hdr);
+        launch_after(k_emit, (unsigned)blocks, kEmitThreads, 0, st, V, w.count, w.gpart, w.offset, w.rec, w.span,
+                     w.rank, w.tile_cur, w.tile_cnt + V.tiles, w.bucket, w.pid, w.hdr);
     }
     // sort each tile's list
     {
         const size_t smem = sizeof(unsigned long long) * kTileSortMax;              // 32 KB: no opt-in needed
-        launch_after(k_tile_sort, (unsigned)V.tiles, kTileSortThreads, smem, st, V, w.tile_order, w.ranges, w.bucket, w.pid,
-                                                                       w.keys_sorted, w.vals_sorted, w.pid_sorted,
-                                                                       w.hdr, &w.hdr->status, cap);
+        launch_after(k_tile_sort, (unsigned)V.tiles, kTileSortThreads, smem, st, V, w.tile_order, w.ranges, w.bucket,
+                     w.pid, w.keys_sorted, w.vals_sorted, w.pid_sorted, w.hdr, &w.hdr->status, cap);
     }
 }
 

@@ -641,8 +641,9 @@ void launch_project_bwd_adam(const Plan& P, const Scenes& S, const float* cams, 
         /* 53 KB (FP32 rows) or 41 KB: above the default 48 KB for FP32 */                                          \
         const size_t smem = (sizeof(float4) * 13 + ShRow<SH>::kRowBytes) * kPbaThreads;                              \
         cudaFuncSetAttribute(k_project_bwd_adam<SH, MO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);   \
-        launch_after(k_project_bwd_adam<SH, MO>, (unsigned)blocks, kPbaThreads, smem, st, P.views, S, cams, w.count, w.offset, \
-                              w.gradrec, A, reinterpret_cast<float4*>(grads_out), w.hdr, (uint32_t)P.cap);         \
+        launch_after(k_project_bwd_adam<SH, MO>, (unsigned)blocks, kPbaThreads, smem, st, P.views, S, cams,         \
+                     w.count, w.offset, w.gradrec, A, reinterpret_cast<float4*>(grads_out), w.hdr,                  \
+                     (uint32_t)P.cap);                                                                              \
     } while (0)
     if (!P.sh_bf16 && !P.mom_bf16) GS_PBA(false, false);
     else if (P.sh_bf16 && P.mom_bf16) GS_PBA(true, true);

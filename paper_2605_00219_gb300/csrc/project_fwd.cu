@@ -179,7 +179,8 @@ void launch_project_fwd(const Plan& P, const Scenes& S, const float* cams, const
     const int T = 256;
     const int64_t blocks = (S.total + T - 1) / T;
     if (blocks == 0) return;
-    launch_after(k_project_fwd, (unsigned)blocks, T, 0, st, P.views, S, cams, w.count, w.tile_cnt, w.rec, w.span, w.rank, w.hdr);
+    launch_after(k_project_fwd, (unsigned)blocks, T, 0, st, P.views, S, cams, w.count, w.tile_cnt, w.rec, w.span,
+                 w.rank, w.hdr);
 }
 
 }  // namespace gs

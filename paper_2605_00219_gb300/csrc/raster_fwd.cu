@@ -328,10 +328,10 @@ void launch_loss_l1(const Plan& P, const WsPtrs& w, const float* image, const fl
     const int64_t blocks = (n + per_block - 1) / per_block;
     if (vec)
         launch_after(k_loss_l1<true>, (unsigned)blocks, kLossThreads, 0, st, image, target, dl, n, 1.0f / (float)n,
-                                                                   w.loss_part, w.hdr);
+                     w.loss_part, w.hdr);
     else
         launch_after(k_loss_l1<false>, (unsigned)blocks, kLossThreads, 0, st, image, target, dl, n, 1.0f / (float)n,
-                                                                    w.loss_part, w.hdr);
+                     w.loss_part, w.hdr);
 }
 
 }  // namespace gs
