@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(kScanThreads) k_densify_decide(int64_t n, cons
                                                                  uint8_t* __restrict__ fate,
                                                                  uint32_t* __restrict__ part)
 {
+    if (!after_previous()) return;
     __shared__ unsigned long long ws[kScanThreads / 32];
     const int64_t base = (int64_t)blockIdx.x * kScanBlock;
     unsigned long long sum = 0;
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(kScanThreads) k_densify_decide(int64_t n, cons
 __global__ void __launch_bounds__(1024) k_densify_scan(int64_t blocks, uint32_t* __restrict__ part,
                                                        int64_t* __restrict__ counts)
 {
+    if (!after_previous()) return;
     __shared__ uint32_t ws[32];
     __shared__ uint32_t tot[3];
     for (int k = 0; k < 3; k++) {
@@ -142,6 +144,7 @@ __global__ void __launch_bounds__(kScanThreads) k_densify_index(const uint8_t* _
                                                                 const int64_t* __restrict__ counts,
                                                                 uint32_t* __restrict__ src)
 {
+    if (!after_previous()) return;
     static_assert(kScanItems == 8, "eight fates in one 64-bit load");
     __shared__ unsigned long long ws[kScanThreads / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -188,6 +191,7 @@ __global__ void __launch_bounds__(256) k_densify_apply(SceneDesc in, SceneDesc o
                                                        const int64_t* __restrict__ counts,
                                                        const float* __restrict__ eps, float factor)
 {
+    if (!after_previous()) return;
     const int64_t n = in.n, m = out.n;
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= m || counts[3] != m) return;   // wrong output size: write nothing
@@ -319,10 +323,10 @@ gs_status gs_densify_count(const gs_scene_buf* scene, int32_t storage_flags, con
     K.grow = cfg->grow != 0;
     K.prune_big = cfg->prune_big != 0;
     const unsigned blocks = (unsigned)ds_blocks(n);
-    k_densify_decide<<<blocks, kScanThreads, 0, st>>>(n, static_cast<const float4*>(scene->geom),
-                                                      static_cast<const float2*>(scene->stats), K, d.fate, d.part);
-    k_densify_scan<<<1, 1024, 0, st>>>(blocks, d.part, d.counts);
-    k_densify_index<<<blocks, kScanThreads, 0, st>>>(d.fate, d.part, d.counts, d.src);
+    launch_after(k_densify_decide, blocks, kScanThreads, 0, st, n, static_cast<const float4*>(scene->geom),
+                 static_cast<const float2*>(scene->stats), K, d.fate, d.part);
+    launch_after(k_densify_scan, 1, 1024, 0, st, blocks, d.part, d.counts);
+    launch_after(k_densify_index, blocks, kScanThreads, 0, st, d.fate, d.part, d.counts, d.src);
     return ds_launch_status();
 }
 
@@ -346,7 +350,7 @@ gs_status gs_densify_apply(const gs_scene_buf* in, int32_t storage_flags, const 
     const SceneDesc si = ds_scene(*in), so = ds_scene(*out);
     const dim3 grid((unsigned)((so.n + 255) / 256), 4);
     const bool sh16 = storage_flags & GS_STORE_SH_BF16, mom16 = storage_flags & GS_STORE_MOMENTS_BF16;
-#define GS_DA(A, B) k_densify_apply<A, B><<<grid, 256, 0, st>>>(si, so, d.src, d.counts, eps, cfg->split_factor)
+#define GS_DA(A, B) launch_after(k_densify_apply<A, B>, grid, 256, 0, st, si, so, d.src, d.counts, eps, cfg->split_factor)
     if (sh16 && mom16) GS_DA(true, true);
     else if (sh16) GS_DA(true, false);
     else if (mom16) GS_DA(false, true);

@@ -13,7 +13,7 @@ namespace gs {
 // Launch of a kernel that starts with after_previous(): programmatic dependent launch,
 // which hides the launch of a kernel behind the end of the one before it in the stream
 // (2,000 Gaussians, eleven launches: 94 -> 72 us a step; 200k, 720p: a render 153 -> 143
-// us).  Not under capture: a graph's plain edges cost less than the waiting blocks do
+// us; a densification of 3M: 486 -> 477 us).  Not under capture: a graph's plain edges cost less than the waiting blocks do
 // (200k, 720p step 313 against 325 us; 3M, 4x1080p 6.00 against 6.08 ms; only the
 // smallest graph gains, 71.8 -> 70.1 us).
 template <typename... Params, typename... Args>
