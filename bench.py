@@ -60,14 +60,14 @@ LR = (1.6e-4 * 30.0, 1e-3, 5e-3, 5e-2, 2.5e-3, 2.5e-3 / 20)   # mean lr scaled b
 # 4 x 1920x1080, 16x16 tiles, pixel-parallel raster backward).  Valid only
 # while the kernel sources hash to the recorded prefixes.
 MEASURED_TRAFFIC = {
-    "raster_bwd": (3760561664, {"raster_bwd.cu": "1bd9c982611a3a21"}),
-    "project_bwd_adam": (3303079168, {"project_bwd_adam.cu": "25d756dbe4558831"}),
-    "raster_fwd": (1647618560, {"raster_fwd.cu": "9bbe3a93408bf2b9"}),
-    "project_fwd": (1741351168, {"project_fwd.cu": "b375359fd7001cef"}),
-    "bin_sort": (1483329536, {"bin_sort.cu": "d92d0a747dcb654f"}),
-    "loss_l1": (259586048, {"raster_fwd.cu": "9bbe3a93408bf2b9"}),
+    "raster_bwd": (3668074240, {"raster_bwd.cu": "451fe35151f7af57", "raster_blocks.cuh": "9ccc2f033f711d05"}),
+    "project_bwd_adam": (3303496960, {"project_bwd_adam.cu": "9e2aff8948ac3ca3"}),
+    "raster_fwd": (1564733440, {"raster_fwd.cu": "76752256a575d173", "raster_blocks.cuh": "9ccc2f033f711d05"}),
+    "project_fwd": (1748315904, {"project_fwd.cu": "19efd11f8f5993d6"}),
+    "bin_sort": (1411531776, {"bin_sort.cu": "e7f70d0097040917"}),
+    "loss_l1": (259816448, {"raster_fwd.cu": "76752256a575d173"}),
 }
-TRAFFIC_COMMON = {"gs_device.cuh": "89b3b04643ff706e", "gs_internal.cuh": "9a90b6b319a8d190"}
+TRAFFIC_COMMON = {"gs_device.cuh": "e5e97ebba1642764", "gs_internal.cuh": "306b4b6d4e0dfc7c"}
 
 
 def _measured_traffic(kernel: str, headline: bool):
