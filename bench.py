@@ -60,7 +60,7 @@ LR = (1.6e-4 * 30.0, 1e-3, 5e-3, 5e-2, 2.5e-3, 2.5e-3 / 20)   # mean lr scaled b
 # 4 x 1920x1080, 16x16 tiles, pixel-parallel raster backward).  Valid only
 # while the kernel sources hash to the recorded prefixes.
 MEASURED_TRAFFIC = {
-    "raster_bwd": (3668074240, {"raster_bwd.cu": "451fe35151f7af57", "raster_blocks.cuh": "9ccc2f033f711d05"}),
+    "raster_bwd": (3668074240, {"raster_bwd.cu": "c758c52b920c67b1", "raster_blocks.cuh": "9ccc2f033f711d05"}),
     "project_bwd_adam": (3303496960, {"project_bwd_adam.cu": "9e2aff8948ac3ca3"}),
     "raster_fwd": (1564733440, {"raster_fwd.cu": "76752256a575d173", "raster_blocks.cuh": "9ccc2f033f711d05"}),
     "project_fwd": (1748315904, {"project_fwd.cu": "19efd11f8f5993d6"}),

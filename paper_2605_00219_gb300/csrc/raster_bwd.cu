@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_raster_bwd(Views V, const uint3
 
 // ===========================================================================
 // The same backward with one pixel's sums per lane replaced by groups of 8 or 16
-// lanes that walk 8x4-pixel blocks, two or four pixels per lane.
+// lanes that walk 8x4- or 8x8-pixel blocks, two or four pixels per lane.
 // ===========================================================================
 
 __device__ __forceinline__ float rcp_approx(float x)
@@ -342,8 +342,8 @@ __device__ __forceinline__ int group_sum_index(int lane)
     return ha ? 5 + k : k;
 }
 
-// Walk of 8x4-pixel blocks of a TW x TH tile, GL lanes to a block (32 / GL pixels
-// each).  Every (entry, block) visit sums its nine values over the block's lanes
+// Walk of 8 x BH-pixel blocks of a TW x TH tile, GL lanes to a block (8 BH / GL
+// pixels each).  Every (entry, block) visit sums its nine values over the block's lanes
 // into a shared-memory slot of its own; an entry's slots are consecutive (a prefix
 // sum over the batch of how many blocks each entry's mask holds), and after the
 // batch one thread per entry adds them in block order.  A batch with more visits
@@ -351,6 +351,8 @@ __device__ __forceinline__ int group_sum_index(int lane)
 // pixel per thread (rows y, y + 2; y, y + 1; columns c, c + 4; ...; blocks in
 // order), so the records are the same bits: for needle-shaped Gaussians the
 // projection backward amplifies a last-ulp change of a record up to 1e4-fold.
+// BH = 8 takes the order of two pixels per thread (rows y, y + 4 one after the other,
+// then y, y + 2; ...) for that choice's FP32 records.
 //
 // Issue-bound (73% of issue slots at 20 warps per SM; ALU 55%, FMA 34%, LSU 28%;
 // 3M Gaussians, one 1080p view).  k_raster_bwd_px spends a warp visit per entry and
@@ -365,18 +367,22 @@ __device__ __forceinline__ int group_sum_index(int lane)
 //   GL = 16 (128 entries a batch, 128 threads): 27.1 -> 20.7 us (2,000 Gaussians,
 //     128x128), 209 -> 183 us (400k, 640x360); 64 entries a batch 23.4 / 214 us.
 //     GL = 8 takes 29.0 / 242 us there: too few blocks to hide one block's chain.
-template <int TW, int TH, int GL>
+//   BH = 8, GL = 16 (64 entries a batch): against two pixels per thread of a warp per
+//     8x8 block 0.96 -> 0.82 ms (3M, one 1080p view), 0.139 -> 0.115 (200k, 720p),
+//     38.6 -> 36.2 us (2,000, 128x128); no grid where it was slower.
+template <int TW, int TH, int GL, int BH>
 struct BwdBlocks {
-    static constexpr int kCols = TW / 8, kBlocks = kCols * (TH / 4);
+    static constexpr int kCols = TW / 8, kBlocks = kCols * (TH / BH);
     static constexpr int kThreads = GL * kBlocks;
     static constexpr int kGroups = 32 / GL;                   // blocks per warp
-    static constexpr int kBatch = GL == 8 ? 64 : 128;         // list entries per staged batch
-    static constexpr int kSlots = GL == 8 ? 224 : 384;        // (entry, block) sums of one pass over a batch
-    static constexpr int kBlocksPerSM = (GL == 8 ? 10 : 5) * 256 / (TW * TH);
+    static constexpr int kPix = 8 * BH / GL;                  // pixels per lane
+    static constexpr int kBatch = kPix == 4 ? 64 : 128;       // list entries per staged batch
+    static constexpr int kSlots = BH == 8 ? 160 : GL == 8 ? 224 : 384;   // (entry, block) sums of one pass over a batch
+    static constexpr int kBlocksPerSM = (kPix == 4 ? 10 : 5) * 256 / (TW * TH);
 };
 
-template <int TW, int TH, int GL>
-__global__ void __launch_bounds__(BwdBlocks<TW, TH, GL>::kThreads, BwdBlocks<TW, TH, GL>::kBlocksPerSM)
+template <int TW, int TH, int GL, int BH>
+__global__ void __launch_bounds__(BwdBlocks<TW, TH, GL, BH>::kThreads, BwdBlocks<TW, TH, GL, BH>::kBlocksPerSM)
 k_raster_bwd_blocks(Views V, const uint32_t* __restrict__ order, const uint2* __restrict__ ranges,
                     const uint32_t* __restrict__ vals_sorted, const uint32_t* __restrict__ pid_sorted,
                     const ProjRec* __restrict__ rec, const float* __restrict__ tfinal, const float* __restrict__ bg,
@@ -384,10 +390,10 @@ k_raster_bwd_blocks(Views V, const uint32_t* __restrict__ order, const uint2* __
                     uint32_t* __restrict__ status, uint32_t cap)
 {
     if (!after_previous()) return;
-    using B = BwdBlocks<TW, TH, GL>;
+    using B = BwdBlocks<TW, TH, GL, BH>;
     constexpr int NT = B::kThreads, NC = B::kCols, NB = B::kBlocks, BB = B::kBatch, S = B::kSlots;
     constexpr int NG = B::kGroups;
-    constexpr int H = 16 / GL;                   // packed pixel pairs per lane
+    constexpr int H = B::kPix / 2;               // packed pixel pairs per lane
     constexpr int IPT = (BB + NT - 1) / NT;      // staged entries per thread
     constexpr int kEnt = 48;                     // bytes of a staged entry
     static_assert(BB % 32 == 0 && NB <= S && 36 * (S + NB) < 65536 && kEnt * BB < 65536, "offsets fit 16 bits");
@@ -411,9 +417,9 @@ k_raster_bwd_blocks(Views V, const uint32_t* __restrict__ order, const uint2* __
     const int lt = (int)(gt - vd.tile_base);
     const int ox = (lt % vd.TX) * TW, oy = (lt / vd.TX) * TH;
     // this lane's column and first row; its pixels are the block's four rows
-    // (8 lanes) or rows y and y + 2 (16 lanes)
+    // (8 lanes) or rows y, y + 2, ... (16 lanes)
     const int px = ox + (blk % NC) * 8 + (lane & 7);
-    const int py = oy + (blk / NC) * 4 + (GL == 8 ? 0 : (lane >> 3) & 1);
+    const int py = oy + (blk / NC) * BH + (GL == 8 ? 0 : (lane >> 3) & 1);
     constexpr int RS = GL == 8 ? 1 : 2;          // row step between the lane's pixels
     const uint2 r = range_at(ranges, gt, cap, status);
     const float fx = (float)(px - ox) + 0.5f, fy = (float)(py - oy) + 0.5f;
@@ -509,8 +515,16 @@ k_raster_bwd_blocks(Views V, const uint32_t* __restrict__ order, const uint2* __
                     sSlot[buf][i] = e_next[u];
 #pragma unroll
                     for (int k = 0; k < NB; k++) m |= b + i < smax[k] ? 1u << k : 0u;
-                    m &= block_mask<TW, TH, 8>(qa.x - ((float)ox + 0.5f), qa.y - ((float)oy + 0.5f), qa.z, qa.w, qb.x,
-                                               qb.y);
+                    uint32_t q = block_mask<TW, TH, 8>(qa.x - ((float)ox + 0.5f), qa.y - ((float)oy + 0.5f), qa.z, qa.w,
+                                                       qb.x, qb.y);
+                    if constexpr (BH == 8) {     // two rows of 8x4 blocks are one
+                        q |= q >> NC;
+                        uint32_t f = 0;
+#pragma unroll
+                        for (int y = 0; y < TH / 8; y++) f |= (q >> (2 * NC * y) & ((1u << NC) - 1u)) << (NC * y);
+                        q = f;
+                    }
+                    m &= q;
                 }
                 sM[buf][i] = m;
                 const uint32_t c = __popc(m);
@@ -608,7 +622,7 @@ k_raster_bwd_blocks(Views V, const uint32_t* __restrict__ order, const uint2* __
                 float2 g9[9];         // sums over the lane's pairs
 #pragma unroll
                 for (int h = 0; h < H; h++) {
-                    const float2 dy = f2(pix_offset(fy + (float)(2 * h), a.y), pix_offset(fy + (float)(2 * h + RS), a.y));
+                    const float2 dy = f2(pix_offset(fy + (float)(RS * 2 * h), a.y), pix_offset(fy + (float)(RS * (2 * h + 1)), a.y));
                     const float p0 = pair_power2_y(px2, dy.x, b.x), p1 = pair_power2_y(px2, dy.y, b.x);
                     float2 G = f2(ex2_approx(p0), ex2_approx(p1));
                     float2 as = f2(__fmul_rn(b.y, G.x), __fmul_rn(b.y, G.y));
@@ -645,6 +659,38 @@ k_raster_bwd_blocks(Views V, const uint32_t* __restrict__ order, const uint2* __
                     // moments of dp = dL/dpower; the conic and the constant factors
                     // are applied per entry
                     const float2 dp = mul2(da, as);
+                    if constexpr (BH == 8) {
+                        // the sums of two lanes of k_raster_bwd_px, a pixel after the other
+                        const float2 y = mul2(dy, dp);
+                        if (h == 0) {
+                            g9[0] = dp;
+                            g9[1] = y;
+                            g9[4] = mul2(dy, y);
+                            g9[5] = mul2(da, G);
+                            g9[6] = t6;
+                            g9[7] = t7;
+                            g9[8] = t8;
+                        } else {
+                            g9[0] = fma2(dp, one1, g9[0]);
+                            g9[1] = fma2(y, one1, g9[1]);
+                            g9[4] = fma2(dy, y, g9[4]);
+                            g9[5] = fma2(da, G, g9[5]);
+                            float2 s6 = fma2(wgt, d0[h], g9[6]), s7 = fma2(wgt, d1[h], g9[7]),
+                                   s8 = fma2(wgt, d2[h], g9[8]);
+                            if constexpr (careful) {
+                                s6 = f2(h0 ? s6.x : g9[6].x, h1 ? s6.y : g9[6].y);
+                                s7 = f2(h0 ? s7.x : g9[7].x, h1 ? s7.y : g9[7].y);
+                                s8 = f2(h0 ? s8.x : g9[8].x, h1 ? s8.y : g9[8].y);
+                            }
+                            g9[6] = s6;
+                            g9[7] = s7;
+                            g9[8] = s8;
+                            g9[0] = mul2(g9[0], dx2);
+                            g9[2] = mul2(dx2, g9[0]);
+                            g9[3] = mul2(dx2, g9[1]);
+                        }
+                        continue;
+                    }
                     float2 t[9];
                     t[0] = mul2(dp, dx2);
                     t[1] = mul2(dy, dp);
@@ -758,8 +804,8 @@ void launch_raster_bwd(const Plan& P, const WsPtrs& w, const float* image, const
 //
 // One CTA per tile, one, two or four pixels per thread, each warp an 8x4, 8x8 or
 // 8x16 pixel block (so a small Gaussian touches few warps).  This form now runs
-// for 8x8 tiles, for two pixels per thread with FP32 moments and for four; the
-// others walk blocks by lane groups (k_raster_bwd_blocks, below).  Every pixel walks its own list prefix
+// for 8x8 tiles and for four pixels per thread; the others walk blocks by lane groups
+// (k_raster_bwd_blocks).  Every pixel walks its own list prefix
 // back to front from its last blended entry: T before an entry is recovered
 // by a compensated division of T after it by (1 - alpha) (div_one_minus:
 // hardware reciprocal, exact remainder, carried low part), and the colour
@@ -1061,30 +1107,31 @@ void launch_raster_bwd_px(const Plan& P, const WsPtrs& w, const float* bg, const
     launch_after(k_raster_bwd_px<BS, TW, PPT>, grid, BS, 0, st, V, w.tile_order, w.ranges, w.vals_sorted,    \
                  w.pid_sorted, w.rec, w.tfinal, bg, dl, w.nlast, w.gradrec, &w.hdr->status,                  \
                  (uint32_t)P.cap)
-#define GS_RBB(TW, TH, GL)                                                                                   \
-    launch_after(k_raster_bwd_blocks<TW, TH, GL>, grid, BwdBlocks<TW, TH, GL>::kThreads, 0, st, V,           \
+#define GS_RBB(TW, TH, GL, BH)                                                                                   \
+    launch_after(k_raster_bwd_blocks<TW, TH, GL, BH>, grid, BwdBlocks<TW, TH, GL, BH>::kThreads, 0, st, V,         \
                  w.tile_order, w.ranges, w.vals_sorted, w.pid_sorted, w.rec, w.tfinal, bg, dl, w.nlast,      \
                  w.gradrec, &w.hdr->status, (uint32_t)P.cap)
     // 16-wide tiles with one pixel per thread (the default) walk 8x4 blocks,
     // and so do two pixels per thread with BF16 moments: their stored rounding
-    // (4e-3) hides the other summation order, which FP32 moments keep.  Four
+    // (4e-3) hides the other summation order, which FP32 moments keep (8x8 blocks:
+    // 0.82 against 0.69 ms at 3M, one 1080p view).  Four
     // visits per warp (GL = 8) need two waves of resident blocks to hide a
     // tile's chain: 2,040 tiles 98.9 us against 83.1 us for GL = 16, 3,600 tiles
     // 100 / 114 us (200k) and 252 / 223 us (1M, sparser), 5,700 tiles 252 / 294 us.
     const bool blocks = ppt == 1 || (ppt == 2 && P.mom_bf16);
-    const bool full = V.tiles >= 2 * (int64_t)P.sm_count * BwdBlocks<16, 16, 8>::kBlocksPerSM * 256 / (V.tw * V.th);
+    const bool full = V.tiles >= 2 * (int64_t)P.sm_count * BwdBlocks<16, 16, 8, 4>::kBlocksPerSM * 256 / (V.tw * V.th);
     if (V.tw == 8) {
         if (ppt == 1) GS_RBP(64, 8, 1);
         else GS_RBP(32, 8, 2);
     } else if (V.th == 16) {
-        if (blocks && full) GS_RBB(16, 16, 8);
-        else if (blocks) GS_RBB(16, 16, 16);
-        else if (ppt == 2) GS_RBP(128, 16, 2);
+        if (blocks && full) GS_RBB(16, 16, 8, 4);
+        else if (blocks) GS_RBB(16, 16, 16, 4);
+        else if (ppt == 2) GS_RBB(16, 16, 16, 8);
         else GS_RBP(64, 16, 4);
     } else {
-        if (blocks && full) GS_RBB(16, 32, 8);
-        else if (blocks) GS_RBB(16, 32, 16);
-        else if (ppt == 2) GS_RBP(256, 16, 2);
+        if (blocks && full) GS_RBB(16, 32, 8, 4);
+        else if (blocks) GS_RBB(16, 32, 16, 4);
+        else if (ppt == 2) GS_RBB(16, 32, 16, 8);
         else GS_RBP(128, 16, 4);
     }
 #undef GS_RBP
