@@ -1,4 +1,4 @@
-"""The L1 + SSIM kernel at the edges of its 32x31 tiles and their 10-pixel
+"""The L1 + SSIM kernel at the edges of 32x31 and 16x16 tiles and their 10-pixel
 halos, against the FP64 oracle, at the tolerances of test_gpu_ssim: views one
 pixel below, at and above a tile and a tile plus its halo, several views in one
 launch, masked and not; and a non-finite pixel, which reaches the gradients of
