@@ -88,8 +88,15 @@ class _GSRender(torch.autograd.Function):
         (image,) = ctx.saved_tensors
         dl = grad_image.contiguous().float()
         gsstep.gs_raster_bwd(r.plan, r.ws, image, dl)
-        # the library writes each scene's gradients in the layout and type of its
-        # stored tensors
-        grads = [(torch.empty_like(b.geom), torch.empty_like(b.sh)) for b in ctx.bufs]
+        # the library writes each scene's gradients in the plan's storage layout,
+        # whatever the scene's tensors are; autograd refuses another shape
+        grads = [(torch.empty((3, b.n, 4), dtype=torch.float32, device=r.device),
+                  torch.empty((6, b.n, 8), dtype=torch.bfloat16, device=r.device) if r.sh_bf16 else
+                  torch.empty((12, b.n, 4), dtype=torch.float32, device=r.device)) for b in ctx.bufs]
         gsstep.gs_project_bwd_grads(r.plan, r.ws, ctx.bufs, r.cams, grads)
-        return (None, *(t for pair in grads for t in pair))
+        out = [None]
+        for b, (dgeom, dsh) in zip(ctx.bufs, grads):
+            if r.sh_bf16 and b.sh.dtype != torch.bfloat16:      # in the layout of other types
+                dsh = dsh.float().reshape(6, b.n, 2, 4).permute(0, 2, 1, 3).reshape(12, b.n, 4)
+            out += [dgeom, dsh]
+        return tuple(out)
