@@ -359,8 +359,8 @@ __device__ __forceinline__ int group_sum_index(int lane)
 // 8x4 block (2.45 an entry) with a quarter of the lanes blending; here a warp
 // iteration serves four (GL = 8: 0.68 an entry) or two (GL = 16: 1.16) visits, and
 // the packed operations both pixels of a pair.  The walk without clamps and guards
-// (no entry of the batch near alpha 0.99, everything finite) saves 26 of about 215
-// instructions: 2.80 -> 2.66 ms.
+// (no entry of the batch near alpha 0.99, no value so large that a product may
+// overflow) saves 26 of about 215 instructions: 2.80 -> 2.66 ms.
 //   GL = 8 (64 entries a batch, 10 blocks of 64 threads per SM): 1.17 -> 0.69 ms
 //     (3M, one 1080p view, FP32), 4.67 -> 2.66 ms (four views), 0.174 -> 0.100 ms
 //     (200k, 720p).  9 / 11 blocks per SM 2.72 / 2.72 ms.
@@ -370,6 +370,10 @@ __device__ __forceinline__ int group_sum_index(int lane)
 //   BH = 8, GL = 16 (64 entries a batch): against two pixels per thread of a warp per
 //     8x8 block 0.96 -> 0.82 ms (3M, one 1080p view), 0.139 -> 0.115 (200k, 720p),
 //     38.6 -> 36.2 us (2,000, 128x128); no grid where it was slower.
+// Colours and loss gradients up to this size have finite products and sums, which the
+// walk without guards multiplies by zero for the pixels that do not blend an entry.
+constexpr float kTame = 1e15f;
+
 template <int TW, int TH, int GL, int BH>
 struct BwdBlocks {
     static constexpr int kCols = TW / 8, kBlocks = kCols * (TH / BH);
@@ -404,7 +408,7 @@ k_raster_bwd_blocks(Views V, const uint32_t* __restrict__ order, const uint2* __
     __shared__ float sQ[2][3][BB];           // conic a, b, c
     __shared__ uint32_t sM[2][BB], sBase[2][BB], sSlot[2][BB];
     // slots of each run of 32 entries; bit 31: an entry's alpha may reach the
-    // 0.99 clamp, or a colour or gradient is not finite
+    // 0.99 clamp, or a colour or gradient is beyond kTame
     __shared__ uint32_t sTot[2][BB / 32];
     __shared__ uint32_t slist[NB][BB + 2];   // entry's byte offset | slot's byte offset << 16
     __shared__ float part[S + NB][9];        // the last NB slots take the stand-in's sums
@@ -437,7 +441,8 @@ k_raster_bwd_blocks(Views V, const uint32_t* __restrict__ order, const uint2* __
     const float2 one1 = f2(one1f, one1f);
     float2 Th[H], Tl[H], nU[H], d0[H], d1[H], d2[H];
     int nl[2 * H];
-    bool odd = false;            // a pixel of the tile has a non-finite dL/dC
+    // a pixel of the tile has a dL/dC, or the background a colour, beyond kTame
+    bool odd = bg && !(fabsf(bg[0]) <= kTame && fabsf(bg[1]) <= kTame && fabsf(bg[2]) <= kTame);
     {
         float t[2 * H], e0[2 * H], e1[2 * H], e2[2 * H], u[2 * H];
 #pragma unroll
@@ -448,7 +453,7 @@ k_raster_bwd_blocks(Views V, const uint32_t* __restrict__ order, const uint2* __
                 nl[k] = (int)nlast[pix];
                 t[k] = tfinal[pix];
                 e0[k] = dl[3 * pix]; e1[k] = dl[3 * pix + 1]; e2[k] = dl[3 * pix + 2];
-                odd |= !(isfinite(e0[k]) && isfinite(e1[k]) && isfinite(e2[k]));
+                odd |= !(fabsf(e0[k]) <= kTame && fabsf(e1[k]) <= kTame && fabsf(e2[k]) <= kTame);
                 if (bg) u[k] = t[k] * fmaf(e0[k], bg[0], fmaf(e1[k], bg[1], e2[k] * bg[2]));
             }
         }
@@ -508,7 +513,7 @@ k_raster_bwd_blocks(Views V, const uint32_t* __restrict__ order, const uint2* __
                     // exponent stays below 1e-6: o 2^p < 0.99 at every pixel
                     const float ac = qa.z * qb.x;
                     flag = odd || !(qb.y <= 0.98f) || !(ac < 1e4f * (ac - qa.w * qa.w)) ||
-                           !(isfinite(qb.z) && isfinite(qb.w) && isfinite(qc.x));
+                           !(fabsf(qb.z) <= kTame && fabsf(qb.w) <= kTame && fabsf(qc.x) <= kTame);
                     sQ[buf][0][i] = qa.z;
                     sQ[buf][1][i] = qa.w;
                     sQ[buf][2][i] = qb.x;
