@@ -15,6 +15,7 @@
 // call left in it; the counter is cleared before every launch.  Calls whose
 // executions overlap on the GPU (different streams, no ordering between
 // them) race on the array and must not be issued.
+#include <cfloat>
 #include <mutex>
 
 #include "gs_internal.cuh"
@@ -108,8 +109,9 @@ __global__ void __launch_bounds__(kNaThreads) k_loss_l1_noalloc(const float* __r
                 }
             }
         }
+        // (an infinite total has no error term: infinity - infinity)
         const float y = t - comp, u = s + y;
-        comp = (u - s) - y;
+        comp = u <= FLT_MAX ? (u - s) - y : 0.f;
         s = u;
     }
 #pragma unroll
@@ -127,18 +129,14 @@ __global__ void __launch_bounds__(kNaThreads) k_loss_l1_noalloc(const float* __r
     if (!is_last) return;
     __threadfence();
     // the blocks' sums as unevaluated pairs (hi, lo), so that the last levels,
-    // at the total's magnitude, round once
+    // at the total's magnitude, round once (lo stays finite when hi is not)
     float hi = 0.f, lo = 0.f;
-    for (unsigned i = threadIdx.x; i < gridDim.x; i += kNaThreads) {
-        float e;
-        gs::two_sum(hi, ((volatile float*)part)[i], hi, e);
-        lo += e;
-    }
     auto add = [&](float h2, float l2) {
         float e;
         gs::two_sum(hi, h2, hi, e);
-        lo += l2 + e;
+        lo += l2 + (hi <= FLT_MAX ? e : 0.f);
     };
+    for (unsigned i = threadIdx.x; i < gridDim.x; i += kNaThreads) add(((volatile float*)part)[i], 0.f);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const float h2 = __shfl_down_sync(0xffffffffu, hi, o), l2 = __shfl_down_sync(0xffffffffu, lo, o);
