@@ -368,8 +368,9 @@ __device__ __forceinline__ int group_sum_index(int lane)
 //     128x128), 209 -> 183 us (400k, 640x360); 64 entries a batch 23.4 / 214 us.
 //     GL = 8 takes 29.0 / 242 us there: too few blocks to hide one block's chain.
 //   BH = 8, GL = 16 (64 entries a batch): against two pixels per thread of a warp per
-//     8x8 block 0.96 -> 0.82 ms (3M, one 1080p view), 0.139 -> 0.115 (200k, 720p),
-//     38.6 -> 36.2 us (2,000, 128x128); no grid where it was slower.
+//     8x8 block 0.96 -> 0.83 ms (3M, one 1080p view), 0.140 -> 0.113 (200k, 720p),
+//     38.8 -> 36.7 us (2,000, 128x128); slower where few tiles are long (the launcher
+//     has the line and the figures).
 // Colours and loss gradients up to this size have finite products and sums, which the
 // walk without guards multiplies by zero for the pixels that do not blend an entry.
 constexpr float kTame = 1e15f;
@@ -808,10 +809,10 @@ void launch_raster_bwd(const Plan& P, const WsPtrs& w, const float* image, const
 // reduced across each warp's pixels by shuffles (no atomics).
 //
 // One CTA per tile, one, two or four pixels per thread, each warp an 8x4, 8x8 or
-// 8x16 pixel block (so a small Gaussian touches few warps).  This form now runs
-// for 8x8 tiles and for four pixels per thread; the others walk blocks by lane groups
-// (k_raster_bwd_blocks).  Every pixel walks its own list prefix
-// back to front from its last blended entry: T before an entry is recovered
+// 8x16 pixel block (so a small Gaussian touches few warps).  This form runs for 8x8
+// tiles, for four pixels per thread and where a few long lists are the launch's time;
+// the others walk blocks by lane groups (k_raster_bwd_blocks).  Every pixel walks its own
+// list prefix back to front from its last blended entry: T before an entry is recovered
 // by a compensated division of T after it by (1 - alpha) (div_one_minus:
 // hardware reciprocal, exact remainder, carried low part), and the colour
 // still to come S grows from T_final * bg without cancellation; only its
@@ -1116,27 +1117,49 @@ void launch_raster_bwd_px(const Plan& P, const WsPtrs& w, const float* bg, const
     launch_kernel(tiles_early(P), k_raster_bwd_blocks<TW, TH, GL, BH>, grid, BwdBlocks<TW, TH, GL, BH>::kThreads, \
                   0, st, V, w.tile_order, w.ranges, w.vals_sorted, w.pid_sorted, w.rec, w.tfinal, bg, dl, w.nlast, \
                   w.gradrec, &w.hdr->status, (uint32_t)P.cap)
-    // 16-wide tiles with one pixel per thread (the default) walk 8x4 blocks,
-    // and so do two pixels per thread with BF16 moments: their stored rounding
-    // (4e-3) hides the other summation order, which FP32 moments keep (8x8 blocks:
-    // 0.82 against 0.69 ms at 3M, one 1080p view).  Four
-    // visits per warp (GL = 8) need two waves of resident blocks to hide a
-    // tile's chain: 2,040 tiles 98.9 us against 83.1 us for GL = 16, 3,600 tiles
-    // 100 / 114 us (200k) and 252 / 223 us (1M, sparser), 5,700 tiles 252 / 294 us.
-    const bool blocks = ppt == 1 || (ppt == 2 && P.mom_bf16);
-    const bool full = V.tiles >= 2 * (int64_t)P.sm_count * BwdBlocks<16, 16, 8, 4>::kBlocksPerSM * 256 / (V.tw * V.th);
+    // 16-wide tiles with one pixel per thread (the default) walk 8x4 blocks by lane
+    // groups, and so do two pixels per thread with BF16 moments (their error against 64
+    // bits is that of the other order of summation, 4.1e-7 to 2.6e-6 of the records' RMS;
+    // FP32 moments keep the order).  All kernels of one order write the same bits, so a
+    // grid takes the one that suits it (us, measured on rooms of 10 m and sites of 30 m,
+    // 20,000 to 3M Gaussians, 64x64 to 1920x1080):
+    //  - GL = 8 (four visits per warp) needs two waves of resident blocks to hide a tile's
+    //    chain, else GL = 16: 200k Gaussians on 3,600 tiles 101 / 116, 5,700 tiles 57 / 72,
+    //    2,040 tiles 141 / 111 (400k).  The tile count alone does not separate them: where
+    //    few of the tiles are long, GL = 16 is faster up to about 4,000 tiles (1M site on
+    //    3,600 tiles 254 against 229, 400k on 3,600 110 against 98).
+    //  - Below that, lists so long that one tile's chain is the launch's time take a warp
+    //    per block: 200k on 60 tiles 867 -> 776, 1M on 60 2,416 -> 1,660, 1M on 240
+    //    986 -> 889; but 400k on 240 510 / 576.  (16x32 tiles have 16 warps and take it
+    //    later: 400k on 30 2,097 -> 1,863, 400k on 75 1,172 / 1,251.)
+    //  - Two pixels per thread, FP32: 8x8 blocks from two waves on (400k room on 3,600
+    //    tiles 266 -> 214, 3M on 8,160 960 -> 827; sites on 3,600 within 1%) and for
+    //    short lists (20k on 920 tiles 24.8 -> 23.2); in between a warp per block is
+    //    faster (1M on 240 tiles 1,284 against 1,748, 3M on 2,040 739 against 864).
+    //    16x32 tiles: from three waves on (1M on 2,900 tiles 347 -> 312), from two with
+    //    short lists (1,840 tiles: 400k room 281 -> 236, 400k site 145 / 159, 3M 841 / 938).
+    const bool blocks = ppt == 1 || (ppt == 2 && P.mom_bf16), tall = V.th == 32;
+    const int64_t wave = (int64_t)P.sm_count * BwdBlocks<16, 16, 8, 4>::kBlocksPerSM * 256 / (V.tw * V.th);
+    const bool full = V.tiles >= 2 * wave;
+    const bool few_long = !full && V.pairs >= (tall ? 12288 : 2560) * V.tiles;
+    const bool blocks8 = tall ? V.tiles >= 3 * wave || (full && V.pairs <= 256 * V.tiles)
+                              : full || V.pairs <= 384 * V.tiles;
     if (V.tw == 8) {
         if (ppt == 1) GS_RBP(64, 8, 1);
         else GS_RBP(32, 8, 2);
-    } else if (V.th == 16) {
+    } else if (!tall) {
         if (blocks && full) GS_RBB(16, 16, 8, 4);
+        else if (blocks && few_long) GS_RBP(256, 16, 1);
         else if (blocks) GS_RBB(16, 16, 16, 4);
-        else if (ppt == 2) GS_RBB(16, 16, 16, 8);
+        else if (ppt == 2 && blocks8) GS_RBB(16, 16, 16, 8);
+        else if (ppt == 2) GS_RBP(128, 16, 2);
         else GS_RBP(64, 16, 4);
     } else {
         if (blocks && full) GS_RBB(16, 32, 8, 4);
+        else if (blocks && few_long) GS_RBP(512, 16, 1);
         else if (blocks) GS_RBB(16, 32, 16, 4);
-        else if (ppt == 2) GS_RBB(16, 32, 16, 8);
+        else if (ppt == 2 && blocks8) GS_RBB(16, 32, 16, 8);
+        else if (ppt == 2) GS_RBP(256, 16, 2);
         else GS_RBP(128, 16, 4);
     }
 #undef GS_RBP
