@@ -996,8 +996,8 @@ void launch_bin_sort(const Plan& P, const WsPtrs& w, cudaStream_t st)
     // sort each tile's list
     {
         const size_t smem = sizeof(unsigned long long) * kTileSortMax;              // 32 KB: no opt-in needed
-        launch_kernel(tiles_early(P), k_tile_sort, (unsigned)V.tiles, kTileSortThreads, smem, st, V, w.tile_order,
-                      w.ranges, w.bucket, w.pid, w.keys_sorted, w.vals_sorted, w.pid_sorted, w.hdr, &w.hdr->status, cap);
+        launch_after(k_tile_sort, (unsigned)V.tiles, kTileSortThreads, smem, st, V, w.tile_order, w.ranges, w.bucket,
+                     w.pid, w.keys_sorted, w.vals_sorted, w.pid_sorted, w.hdr, &w.hdr->status, cap);
     }
 }
 

@@ -10,10 +10,12 @@
 
 namespace gs {
 
-// early: by programmatic dependent launch, unless the stream is being captured.
+// Launch of a kernel that starts with after_previous(): programmatic dependent launch,
+// which hides the launch of a kernel behind the end of the one before it in the stream
+// (2,000 Gaussians, eleven launches: 94 -> 70 us a step; 200k, 720p: a render 153 -> 140
+// us; a densification of 3M: 486 -> 475 us).  A graph's edges stay plain.
 template <typename... Params, typename... Args>
-inline void launch_kernel(bool early, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                          Args&&... args)
+inline void launch_after(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args)
 {
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -23,25 +25,11 @@ inline void launch_kernel(bool early, void (*kernel)(Params...), dim3 grid, dim3
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    if (early) {
-        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-        cudaStreamIsCapturing(st, &capture);
-        cfg.attrs = &at;
-        cfg.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
-    }
+    cfg.attrs = &at;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(st, &capture);
+    cfg.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-
-// Launch of a kernel that starts with after_previous(): programmatic dependent launch,
-// which hides the launch of a kernel behind the end of the one before it in the stream
-// (2,000 Gaussians, eleven launches: 94 -> 72 us a step; a densification of 3M:
-// 486 -> 477 us).  Not under capture: a graph's plain edges cost less than the
-// waiting blocks do (200k, 720p step 313 against 325 us; 3M, 4x1080p 6.00 against
-// 6.08 ms; only the smallest graph gains, 71.8 -> 70.1 us).
-template <typename... Params, typename... Args>
-inline void launch_after(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args)
-{
-    launch_kernel(true, kernel, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
 // Intersection capacity granule (the capacity is rounded up to it).
@@ -116,20 +104,6 @@ inline int tile_ppt(const Plan& P)
 {
     const int np = P.views.tw * P.views.th;
     return P.tuning.threads_per_tile > 0 ? np / P.tuning.threads_per_tile : 1;
-}
-
-// Whether the kernels of one block per tile (tile sort, raster forward and backward) are
-// launched early.  Early blocks take the places that the kernel before leaves first,
-// three to an SM while others are still busy; a few long tiles then share an SM for the
-// whole launch (1M Gaussians, 480x270: a render 754 against 616 us, a step 1,654 against
-// 1,440; 3M, 1280x720: 1,793 against 1,723).  Light tiles gain the launches' latency
-// (20,000, 640x360: a step 73 against 78 us; 100,000, 1280x720: 191 / 193), and so do
-// grids of several waves, whatever the tiles hold (200,000, 1920x1080: 449 / 458 us; 3M:
-// 2,193 / 2,204).  In between, 32 Gaussians a tile: 65,000 on 2,040 tiles 129 / 129 us,
-// on 920 126 / 126, on 240 216 / 203.
-inline bool tiles_early(const Plan& P)
-{
-    return P.views.tiles >= 4096 || P.views.pairs <= std::max<int64_t>(32768, 32 * P.views.tiles);
 }
 
 Scenes make_scenes(const Plan& P, const gs_scene_buf* scenes);

@@ -793,8 +793,8 @@ void launch_raster_bwd(const Plan& P, const WsPtrs& w, const float* image, const
             cudaFuncSetAttribute(k_raster_bwd<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb);   \
             attr_set = true;                                                                                \
         }                                                                                                   \
-        launch_kernel(tiles_early(P), k_raster_bwd<NP>, grid, kBwdThreads, sb, st, V, w.tile_order, w.ranges, \
-                      w.vals_sorted, w.pid_sorted, w.rec, image, dl, w.nlast, w.gradrec, fixed);            \
+        launch_after(k_raster_bwd<NP>, grid, kBwdThreads, sb, st, V, w.tile_order, w.ranges, w.vals_sorted, \
+                     w.pid_sorted, w.rec, image, dl, w.nlast, w.gradrec, fixed);                            \
     } while (0)
     if (np == 64) GS_RB(64);
     else if (np == 256) GS_RB(256);
@@ -1110,13 +1110,13 @@ void launch_raster_bwd_px(const Plan& P, const WsPtrs& w, const float* bg, const
     const unsigned grid = (unsigned)V.tiles;
     const int ppt = tile_ppt(P);
 #define GS_RBP(BS, TW, PPT)                                                                                  \
-    launch_kernel(tiles_early(P), k_raster_bwd_px<BS, TW, PPT>, grid, BS, 0, st, V, w.tile_order, w.ranges,  \
-                  w.vals_sorted, w.pid_sorted, w.rec, w.tfinal, bg, dl, w.nlast, w.gradrec, &w.hdr->status,  \
-                  (uint32_t)P.cap)
+    launch_after(k_raster_bwd_px<BS, TW, PPT>, grid, BS, 0, st, V, w.tile_order, w.ranges, w.vals_sorted,    \
+                 w.pid_sorted, w.rec, w.tfinal, bg, dl, w.nlast, w.gradrec, &w.hdr->status,                  \
+                 (uint32_t)P.cap)
 #define GS_RBB(TW, TH, GL, BH)                                                                                   \
-    launch_kernel(tiles_early(P), k_raster_bwd_blocks<TW, TH, GL, BH>, grid, BwdBlocks<TW, TH, GL, BH>::kThreads, \
-                  0, st, V, w.tile_order, w.ranges, w.vals_sorted, w.pid_sorted, w.rec, w.tfinal, bg, dl, w.nlast, \
-                  w.gradrec, &w.hdr->status, (uint32_t)P.cap)
+    launch_after(k_raster_bwd_blocks<TW, TH, GL, BH>, grid, BwdBlocks<TW, TH, GL, BH>::kThreads, 0, st, V,         \
+                 w.tile_order, w.ranges, w.vals_sorted, w.pid_sorted, w.rec, w.tfinal, bg, dl, w.nlast,      \
+                 w.gradrec, &w.hdr->status, (uint32_t)P.cap)
     // 16-wide tiles with one pixel per thread (the default) walk 8x4 blocks by lane
     // groups, and so do two pixels per thread with BF16 moments (their error against 64
     // bits is that of the other order of summation, 4.1e-7 to 2.6e-6 of the records' RMS;

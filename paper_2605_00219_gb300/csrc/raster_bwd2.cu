@@ -332,8 +332,8 @@ void launch_raster_bwd2(const Plan& P, const WsPtrs& w, const float* bg, const f
             cudaFuncSetAttribute(k_raster_bwd2<BS, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb); \
             attr_set = true;                                                                                  \
         }                                                                                                     \
-        launch_kernel(tiles_early(P), k_raster_bwd2<BS, TW>, grid, BS, sb, st, V, w.tile_order, w.ranges,     \
-                      w.vals_sorted, w.pid_sorted, w.rec, w.tfinal, bg, dl, w.nlast, w.gradrec);              \
+        launch_after(k_raster_bwd2<BS, TW>, grid, BS, sb, st, V, w.tile_order, w.ranges, w.vals_sorted,       \
+                     w.pid_sorted, w.rec, w.tfinal, bg, dl, w.nlast, w.gradrec);                              \
     } while (0)
     if (V.tw == 8) GS_RB2(64, 8);
     else if (V.th == 16) GS_RB2(256, 16);

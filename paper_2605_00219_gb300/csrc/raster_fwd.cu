@@ -219,7 +219,7 @@ void launch_raster_fwd(const Plan& P, const WsPtrs& w, const float* bg, float* i
 {
     const Views& V = P.views;
     const unsigned grid = (unsigned)V.tiles;
-#define GS_RF(TW, TH) launch_kernel(tiles_early(P), k_raster_fwd<TW, TH>, grid, TileBlocks<TW, TH>::kThreads, 0, st,          \
+#define GS_RF(TW, TH) launch_after(k_raster_fwd<TW, TH>, grid, TileBlocks<TW, TH>::kThreads, 0, st,                           \
         V, w.tile_order, w.ranges, w.pid_sorted, w.rec, bg, image, w.tfinal, w.nlast, w.hdr, (uint32_t)P.cap)
     if (V.tw == 8) GS_RF(8, 8);
     else if (V.th == 16) GS_RF(16, 16);
