@@ -32,20 +32,6 @@
 
 namespace gs {
 
-__global__ void k_fill_u32(uint32_t* __restrict__ p, int64_t n, uint32_t value)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = value;
-}
-
-void launch_fill_u32(uint32_t* p, int64_t n, uint32_t value, cudaStream_t st)
-{
-    if (n <= 0) return;
-    int64_t blocks = (n + 255) / 256;
-    if (blocks > 152 * 16) blocks = 152 * 16;
-    k_fill_u32<<<(unsigned)blocks, 256, 0, st>>>(p, n, value);
-}
-
 // ---------------------------------------------------------------------------
 // Emission slots, tile ranges and launch order
 // ---------------------------------------------------------------------------
@@ -468,8 +454,7 @@ __global__ void __launch_bounds__(kEmitThreads, 5) k_emit(Views V, const uint32_
             gm.r2 = cull_r2(rec[kp].b.y);
             gm.mant = ks.x & 0x7FFFFFu;
             gm.valid = 1;
-            uint32_t bands;
-            warp_scanline(gm, V.tw, V.th, kd.TX, kd.TY, bands, [](uint32_t, bool, int, int, int) {}, place);
+            warp_scanline(gm, V.tw, V.th, kd.TX, kd.TY, place);
         } else {
             const bool rows = (ks.x >> 26) & 1u;
             for (uint32_t i = threadIdx.x & 31; i < kcnt; i += 32)
@@ -619,8 +604,9 @@ __device__ void block_merge_sort_smem(unsigned long long* s, int N, const SortGr
 
 // Ascending sort of a warp's 256 keys in registers, lane l holding [8l, 8l + 8):
 // 8 keys by the network, then bitonic merges of run width 8, 16, ... up to `most`
-// keys, which lie in the first most / 8 lanes (each: the mirrored exchange, then halving exchanges, across lanes by shuffles
-// and within a lane in registers).  No shared-memory round trips.
+// keys, which lie in the first most / 8 lanes (each: the mirrored exchange, then halving
+// exchanges, across lanes by shuffles and within a lane in registers).  No shared-memory
+// round trips.
 __device__ __forceinline__ void warp_sort256(uint32_t* r, int lane, int most)
 {
     sort8(r);
@@ -720,8 +706,8 @@ __device__ void merge_level(const Src& src, const Dst& dst, uint32_t s0, uint32_
     }
 }
 
-// The tile sort (longest lists launched first).  Input: the tile's bucket [s0, s1) of (depth code, emission slot) in atomic arrival
-// order.  Output at the same positions: keys_sorted = tile << shift | depth
+// The tile sort (longest lists launched first).  Input: the tile's bucket [s0, s1) of
+// (depth code, emission slot) in atomic arrival order.  Output at the same positions: keys_sorted = tile << shift | depth
 // code, vals_sorted = emission slot, pid_sorted = the slot's pair.
 //
 // A run of n <= IT g.n entries at b, sorted by the group on 32-bit words (depth code,
@@ -738,8 +724,8 @@ __device__ void merge_level(const Src& src, const Dst& dst, uint32_t s0, uint32_
 constexpr int kTieRun = 32;
 
 template <int IT, typename Pair, typename Put>
-__device__ __forceinline__ bool sort_words(const uint2* b, int n, int bits, uint32_t* key, const SortGroup& g, Pair pair,
-                                           Put put)
+__device__ __forceinline__ bool sort_words(const uint2* b, int n, int bits, uint32_t* key, const SortGroup& g,
+                                           Pair pair, Put put)
 {
     const int ib = 32 - __clz((n - 1) | 1);        // bits of the arrival index
     if (bits + ib > 32) return false;

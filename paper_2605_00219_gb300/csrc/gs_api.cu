@@ -99,7 +99,6 @@ static bool plan_build(Plan& P, const int64_t* scene_n, int32_t n_scenes, const 
     V.th = t.tile_h;
     V.n_scenes = n_scenes;
     int64_t pairs = 0, tiles = 0, pixels = 0;
-    int max_bits = 0;
     for (int v = 0; v < n_views; v++) {
         const gs_view& gv = views[v];
         if (gv.width < 1 || gv.height < 1 || gv.width > 16384 || gv.height > 16384) return false;
@@ -116,7 +115,6 @@ static bool plan_build(Plan& P, const int64_t* scene_n, int32_t n_scenes, const 
         const int tb = ceil_log2((int64_t)d.TX * d.TY);
         d.shift = tb >= 9 ? 32 - tb : 23;
         d.drop = tb >= 9 ? tb - 9 : 0;
-        max_bits = std::max(max_bits, tb >= 9 ? 32 : 23 + tb);
         d.pair_base = pairs;
         d.tile_base = tiles;
         d.pix_base = pixels;
@@ -127,7 +125,6 @@ static bool plan_build(Plan& P, const int64_t* scene_n, int32_t n_scenes, const 
     V.pairs = pairs;
     V.tiles = tiles;
     V.pixels = pixels;
-    (void)max_bits;
     {
         int64_t q = 0;
         for (int sc = 0; sc < n_scenes; sc++) {

@@ -454,18 +454,14 @@ __device__ __forceinline__ uint32_t scanline_bands(const BinGeom& g, const ScanL
 
 // The traversal of one pair by a whole warp (every lane with the same g): the
 // lanes take a band each, then the tiles of those bands in order, 32 at a time:
-// emit(i, tile id) for the i-th tile.  first2(k, coord, lo, hi) is called by every
-// lane for the first two bands that meet a tile.  Returns the tiles, and in nb the bands.
-// A lane that walked a footprint of a thousand tiles alone held its block for the
+// emit(i, tile id) for the i-th tile.  A lane that walked a footprint of a thousand tiles alone held its block for the
 // whole kernel's time.
-template <typename First2, typename Emit>
-__device__ __forceinline__ uint32_t warp_scanline(const BinGeom& g, int tw, int th, int TX, int TY, uint32_t& nb,
-                                                  First2 first2, Emit emit)
+template <typename Emit>
+__device__ __forceinline__ void warp_scanline(const BinGeom& g, int tw, int th, int TX, int TY, Emit emit)
 {
     const ScanLine L = scanline_setup(g, tw, th, TX, TY);
     const int lane = threadIdx.x & 31;
     uint32_t count = 0;
-    nb = 0;
     for (int c0 = L.first; c0 <= L.last; c0 += 32) {
         int lo = 0, hi = -1;
         const int c = c0 + lane;
@@ -476,11 +472,6 @@ __device__ __forceinline__ uint32_t warp_scanline(const BinGeom& g, int tw, int 
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
-        }
-        for (uint32_t m = __ballot_sync(0xffffffffu, n != 0u); m && nb < 3u; m &= m - 1u, nb++) {
-            const int k = __ffs(m) - 1;
-            const int l = __shfl_sync(0xffffffffu, lo, k), h = __shfl_sync(0xffffffffu, hi, k);
-            if (nb < 2u) first2(nb, L.rows, c0 + k, l, h);
         }
         const uint32_t total = __shfl_sync(0xffffffffu, x, 31);
         for (uint32_t i0 = 0; i0 < total; i0 += 32) {
@@ -499,7 +490,6 @@ __device__ __forceinline__ uint32_t warp_scanline(const BinGeom& g, int tw, int 
         }
         count += total;
     }
-    return count;
 }
 
 // Tile span of a pair, written by the projection's traversal and read by

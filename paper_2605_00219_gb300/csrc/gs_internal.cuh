@@ -120,7 +120,6 @@ void launch_raster_bwd(const Plan& P, const WsPtrs& w, const float* image, const
 void launch_raster_bwd2(const Plan& P, const WsPtrs& w, const float* bg, const float* dl, cudaStream_t st);
 void launch_project_bwd_adam(const Plan& P, const Scenes& S, const float* cams, const WsPtrs& w,
                              const gs_adam* adam, float* grads_out, cudaStream_t st);
-void launch_fill_u32(uint32_t* p, int64_t n, uint32_t value, cudaStream_t st);
 void launch_ws_init(const Plan& P, const WsPtrs& w, cudaStream_t st);
 void launch_adam_advance(const WsPtrs& w, cudaStream_t st);
 

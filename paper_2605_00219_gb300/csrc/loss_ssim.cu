@@ -186,7 +186,8 @@ __global__ void __launch_bounds__(kSsThreads, kSsCtas)
         }
         const float mc = pix_mask<MASK>(tc);
         if (tid < kSsP)
-            shift[tid] = make_float2(isfinite(ic * mc) ? ic * mc : 0.f, MASK ? target_channel(tc, c) * mc : target_code(tc, c));
+            shift[tid] = make_float2(isfinite(ic * mc) ? ic * mc : 0.f,
+                                     MASK ? target_channel(tc, c) * mc : target_code(tc, c));
 #pragma unroll
         for (int k = 0; k < NR; k++) {
             const int r = r0 + RS * k;

@@ -59,9 +59,9 @@ struct TileBlocks {
 // Conservative mask of the tile's BW x 4 blocks (BW = 4 or 8) that an entry can
 // contribute to; warp w's four blocks are the bits 4w .. 4w + 3 (lane group
 // g = bit 4w + g): 4x4 blocks in quads of 8x8 pixels, 8x4 blocks row by row.
-// (x, y): the mean relative to the centre of the tile's first pixel.  A pair needs d^2 <= r^2 = min(9, 2 ln(255 o)); for each row of blocks
-// the ellipse's extreme x over the row's band gives the first and last block:
-// with h(dy) = sqrt(r^2/a - det dy^2 / a^2) the ellipse spans
+// (x, y): the mean relative to the centre of the tile's first pixel.  A pair needs
+// d^2 <= r^2 = min(9, 2 ln(255 o)); for each row of blocks the ellipse's extreme x over
+// the row's band gives the first and last block: with h(dy) = sqrt(r^2/a - det dy^2 / a^2) the ellipse spans
 // x - (b/a) dy -/+ h(dy), extreme at dy = -/+ ys (the offset of the leftmost /
 // rightmost point) clamped to the band.  Against the box of the ellipse this
 // drops 17% of the (entry, block) visits at the size above and costs about

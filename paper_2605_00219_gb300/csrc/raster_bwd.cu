@@ -628,7 +628,8 @@ k_raster_bwd_blocks(Views V, const uint32_t* __restrict__ order, const uint2* __
                 float2 g9[9];         // sums over the lane's pairs
 #pragma unroll
                 for (int h = 0; h < H; h++) {
-                    const float2 dy = f2(pix_offset(fy + (float)(RS * 2 * h), a.y), pix_offset(fy + (float)(RS * (2 * h + 1)), a.y));
+                    const float2 dy = f2(pix_offset(fy + (float)(RS * 2 * h), a.y),
+                                         pix_offset(fy + (float)(RS * (2 * h + 1)), a.y));
                     const float p0 = pair_power2_y(px2, dy.x, b.x), p1 = pair_power2_y(px2, dy.y, b.x);
                     float2 G = f2(ex2_approx(p0), ex2_approx(p1));
                     float2 as = f2(__fmul_rn(b.y, G.x), __fmul_rn(b.y, G.y));
