@@ -111,11 +111,17 @@ typedef struct {
                                  thread, each warp covering 8 x 8 or 8 x 16
                                  pixels (Sec. 4.2: the scheduler's threads per
                                  tile).  Pixels per thread other than 1 need
-                                 bwd_impl 0.  It selects how the gradient sums
-                                 are formed; the library maps one pixel per
-                                 thread (and two, with BF16 moments) to lane
-                                 groups over 8 x 4 pixel blocks.  The raster
-                                 forward does not depend on it. */
+                                 bwd_impl 0.  It selects in which order the
+                                 gradient sums are formed; which kernel forms
+                                 them is the library's choice by the grid.  On
+                                 16-wide tiles one pixel per thread, and two
+                                 with BF16 moments, are lane groups over 8 x 4
+                                 pixel blocks (a warp per block for few, long
+                                 lists); two with FP32 moments are lane groups
+                                 over 8 x 8 blocks or a warp per block.  8 x 8
+                                 tiles, and four pixels per thread, take a warp
+                                 per block.  The raster forward does not depend
+                                 on it. */
 } gs_tuning;
 
 typedef struct {

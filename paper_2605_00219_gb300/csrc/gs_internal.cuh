@@ -12,7 +12,7 @@ namespace gs {
 
 // Launch of a kernel that starts with after_previous(): programmatic dependent launch,
 // which hides the launch of a kernel behind the end of the one before it in the stream
-// (2,000 Gaussians, eleven launches: 94 -> 70 us a step; 200k, 720p: a render 153 -> 140
+// (2,000 Gaussians, eleven launches: 94 -> 70 us a step; 200k, 1237x822: a render 153 -> 137
 // us; a densification of 3M: 486 -> 475 us).  A graph's edges stay plain.
 template <typename... Params, typename... Args>
 inline void launch_after(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args)
