@@ -60,14 +60,14 @@ LR = (1.6e-4 * 30.0, 1e-3, 5e-3, 5e-2, 2.5e-3, 2.5e-3 / 20)   # mean lr scaled b
 # 4 x 1920x1080, 16x16 tiles, pixel-parallel raster backward).  Valid only
 # while the kernel sources hash to the recorded prefixes.
 MEASURED_TRAFFIC = {
-    "raster_bwd": (3668074240, {"raster_bwd.cu": "c758c52b920c67b1", "raster_blocks.cuh": "9ccc2f033f711d05"}),
-    "project_bwd_adam": (3303496960, {"project_bwd_adam.cu": "9e2aff8948ac3ca3"}),
-    "raster_fwd": (1564733440, {"raster_fwd.cu": "76752256a575d173", "raster_blocks.cuh": "9ccc2f033f711d05"}),
-    "project_fwd": (1748315904, {"project_fwd.cu": "19efd11f8f5993d6"}),
-    "bin_sort": (1411531776, {"bin_sort.cu": "e7f70d0097040917"}),
-    "loss_l1": (259816448, {"raster_fwd.cu": "76752256a575d173"}),
+    "raster_bwd": (3666846976, {"raster_bwd.cu": "665e1dfb07817b1f", "raster_blocks.cuh": "f1ef771177247624"}),
+    "project_bwd_adam": (3303788544, {"project_bwd_adam.cu": "9e2aff8948ac3ca3"}),
+    "raster_fwd": (1564635136, {"raster_fwd.cu": "76752256a575d173", "raster_blocks.cuh": "f1ef771177247624"}),
+    "project_fwd": (1747398400, {"project_fwd.cu": "19efd11f8f5993d6"}),
+    "bin_sort": (1421848832, {"bin_sort.cu": "75eb607fe698136c"}),
+    "loss_l1": (259999232, {"raster_fwd.cu": "76752256a575d173"}),
 }
-TRAFFIC_COMMON = {"gs_device.cuh": "e5e97ebba1642764", "gs_internal.cuh": "306b4b6d4e0dfc7c"}
+TRAFFIC_COMMON = {"gs_device.cuh": "12d5d3243b05b8ef", "gs_internal.cuh": "06f4ab0ac68bf22f"}
 
 
 def _measured_traffic(kernel: str, headline: bool):

